@@ -27,6 +27,7 @@
 #include <stdlib.h>
 
 #include "biot_common.cuh"
+#include "wall_table.cuh"
 
 namespace biot {
 
@@ -312,8 +313,8 @@ struct CollideOut {
 // extra values e in the raw-ring order of RingLayout) and m_s of its eight
 // neighbours; shared by the ring and register forms of the strip sweep, so that
 // both round identically.
-template <typename T, typename TC, int KIND, bool LO, int NE>
-__device__ __forceinline__ CollideOut<T> collide_math(const SweepArgs<T, TC> &a, T m0, T m1, T m2, T m3, T m4,
+template <typename T, int KIND, bool LO, int NE, typename A>
+__device__ __forceinline__ CollideOut<T> collide_math(const A &a, T m0, T m1, T m2, T m3, T m4,
                                                      const T (&e)[NE], T dE, T dW, T dN, T dS, T dNE, T dNW, T dSE,
                                                      T dSW)
 {
@@ -401,7 +402,7 @@ __device__ __forceinline__ void collide_cell(const SweepArgs<T, TC> &a, const Ri
     rg.get_extras(s, c, e);
     const T dE = rg.ms(s, c + 1), dW = rg.ms(s, c - 1), dN = rg.ms(sp, c), dS = rg.ms(sm, c);
     const T dNE = rg.ms(sp, c + 1), dNW = rg.ms(sp, c - 1), dSE = rg.ms(sm, c + 1), dSW = rg.ms(sm, c - 1);
-    const CollideOut<T> o = collide_math<T, TC, KIND, LO, L::NE>(a, q0.x, q0.y, q0.z, rg.ms(s, c), q0.w, e, dE, dW, dN,
+    const CollideOut<T> o = collide_math<T, KIND, LO, L::NE>(a, q0.x, q0.y, q0.z, rg.ms(s, c), q0.w, e, dE, dW, dN,
                                                                  dS, dNE, dNW, dSE, dSW);
 #pragma unroll
     for (int k = 0; k < 8; k++) rg.G(s, k, c) = o.G[k];
@@ -442,8 +443,10 @@ __device__ __forceinline__ PVal<T> pval_from(T g, T smx, T smy, T tx, T ty, T tl
     return v;
 }
 
-template <typename T, bool LO, int W, int KIND, int K>
-__device__ __forceinline__ PVal<T> post_at(const Rings<T, W, KIND, LO> &rg, int s, int c, T tx, T ty, T tlx, T tly)
+// RG: the post-collision data by (slot, column): the rings of a strip or tile, or
+// the rows of a resident level.
+template <typename T, bool LO, int K, typename RG>
+__device__ __forceinline__ PVal<T> post_at(const RG &rg, int s, int c, T tx, T ty, T tlx, T tly)
 {
     constexpr int p = pair_of(K);
     const T smx = pa_x(p) != 0.0 ? rg.MX(s, c) : T(0);
@@ -451,100 +454,95 @@ __device__ __forceinline__ PVal<T> post_at(const Rings<T, W, KIND, LO> &rg, int 
     return pval_from<T, LO, K>(rg.G(s, K, c), smx, smy, tx, ty, tlx, tly);
 }
 
-// Population of direction K arriving at cell (x, y) (ring column c0); sl[0..2]
-// are the slots of rows y-1, y, y+1.
-template <typename T, typename TC, int KIND, bool LO, int W, int K, bool WALL>
-__device__ __forceinline__ PVal<T> pull(const SweepArgs<T, TC> &a, const Rings<T, W, KIND, LO> &rg, int x, int y,
-                                        const int (&sl)[3], int c0, T tx, T ty, T tlx, T tly, bool perx, bool pery)
+// v with its sign flipped where the top bit of `bit` is set (no FP64 instruction:
+// one holds an SM's FP64 unit for 64 cycles).
+__device__ __forceinline__ float flip_sign(float v, unsigned bit)
 {
-    constexpr int cx = ex8(K), cy = ey8(K);
-    const int s0 = sl[1];
-    if (!WALL) return post_at<T, LO, W, KIND, K>(rg, sl[1 - cy], c0 - cx, tx, ty, tlx, tly);
-    const int sx = x - cx, sy = y - cy;
-    const bool outx = !perx && (sx < 0 || sx >= a.nx);
-    const bool outy = !pery && (sy < 0 || sy >= a.ny);
-    if (!outx && !outy) return post_at<T, LO, W, KIND, K>(rg, sl[1 - cy], c0 - cx, tx, ty, tlx, tly);
-    int side = outy ? (sy < 0 ? SIDE_BOTTOM : SIDE_TOP) : (sx < 0 ? SIDE_LEFT : SIDE_RIGHT);
-    if (outy && outx) {
-        // corner: a bounce-back type side wall wins over a mirror top/bottom
-        const int vert = sx < 0 ? SIDE_LEFT : SIDE_RIGHT;
-        if (a.bc[side] == BC_SYMMETRY && a.bc[vert] != BC_SYMMETRY) side = vert;
-    }
-    const int type = a.bc[side];
-    if (type == BC_SYMMETRY) {
-        // mirror image of the ghost source, normal velocity reversed
-        if (outy) {
-            if (outx) return post_at<T, LO, W, KIND, dir8(-cx, -cy)>(rg, s0, c0, tx, ty, tlx, tly);
-            return post_at<T, LO, W, KIND, dir8(cx, -cy)>(rg, s0, c0 - cx, tx, ty, tlx, tly);
-        }
-        return post_at<T, LO, W, KIND, dir8(-cx, cy)>(rg, sl[1 - cy], c0, tx, ty, tlx, tly);
-    }
-    constexpr int kout = opp8(K);
-    const PVal<T> o = post_at<T, LO, W, KIND, kout>(rg, s0, c0, tx, ty, tlx, tly);
-    const bool horiz = (side == SIDE_BOTTOM || side == SIDE_TOP);
-    const int n = horiz ? a.nx : a.ny;
-    PVal<T> v;
-    if (type == BC_NEUMANN) {  // eq. BC:traction
-        v.g = -o.g;
-        v.h = -o.h;
-        v.bx = -o.bx;
-        v.by = -o.by;
-        if (kind_fine(KIND) && a.prof[side]) v.g += T(a.c0h * traction_term(a.prof[side], side, n, x, y, cx, cy));
-        return v;
-    }
-    // BC_DIRICHLET: eq. BC:elasticity, history = previous call's outgoing population
-    if (a.hist_valid) {
-        v.g = a.H[side][3 * (horiz ? x : y) + hslot(side, kout)];
-        v.h = T(0);
-        v.bx = T(0);
-        v.by = T(0);
-    } else {
-        v = o;
-    }
-    if (kind_fine(KIND) && a.prof[side]) v.g += T(dirichlet_term(a.prof[side], side, n, x, y, cx, cy));
-    return v;
+    return __uint_as_float(__float_as_uint(v) ^ (bit & 0x80000000u));
+}
+__device__ __forceinline__ double flip_sign(double v, unsigned bit)
+{
+    return __hiloint2double(__double2hiint(v) ^ (int)(bit & 0x80000000u), __double2loint(v));
 }
 
-// Pair p after streaming: S = g_first + g_second, A = g_first - g_second, each
-// as a small part plus a beta part.  dB = (beta difference) - a_p vanishes
-// exactly away from walls, as does the beta sum.
+// The walls cell (x, y) touches, as an index of the wall table.
+template <typename A>
+__device__ __forceinline__ int wall_cell_index(const A &a, int x, int y, bool perx, bool pery)
+{
+    auto kind = [&](int side) { return a.bc[side] == BC_DIRICHLET && a.hist_valid ? (int)WALL_DIR : a.bc[side]; };
+    const int eL = !perx && x == 0 ? kind(SIDE_LEFT) : 0, eR = !perx && x == a.nx - 1 ? kind(SIDE_RIGHT) : 0;
+    const int eB = !pery && y == 0 ? kind(SIDE_BOTTOM) : 0, eT = !pery && y == a.ny - 1 ? kind(SIDE_TOP) : 0;
+    return wall_index(eL, eR, eB, eT);
+}
+
+// Population of direction K arriving at a wall cell (x, y) (ring column c0), as
+// its descriptor w says (wall_table.cuh); sl[0..2] are the slots of rows y-1, y,
+// y+1.  g and h as in PVal; the beta terms come from the table.
+template <typename T, int KIND, bool LO, int K, typename A, typename RG>
+__device__ __forceinline__ void wall_pull_at(const A &a, const RG &rg, unsigned w, int x, int y, const int (&sl)[3], int c0,
+                                             T tx, T ty, T tlx, T tly, T &g, T &h)
+{
+    constexpr int cx = ex8(K), cy = ey8(K), p = pair_of(K);
+    constexpr int vert = cx > 0 ? SIDE_LEFT : SIDE_RIGHT, hor = cy > 0 ? SIDE_BOTTOM : SIDE_TOP;
+    const int row = (w >> WP_ROW) & 3, s = row == 0 ? sl[0] : row == 1 ? sl[1] : sl[2], c = c0 - 1 + (int)((w >> WP_COL) & 3);
+    g = flip_sign(rg.G(s, w & WP_K, c), w << (31 - WP_SG));
+    T dx = T(0), dy = T(0);
+    if constexpr (cx != 0) {
+        dx = rg.MX(s, c) - tx;
+        if constexpr (LO) dx -= tlx;
+    }
+    if constexpr (cy != 0) {
+        dy = rg.MY(s, c) - ty;
+        if constexpr (LO) dy -= tly;
+    }
+    T q;
+    if constexpr (p == 0) q = mul_rn(T(1.0 / 3.0), dx);
+    else if constexpr (p == 1) q = mul_rn(T(1.0 / 3.0), dy);
+    else q = mul_rn(T(1.0 / 12.0), dy + flip_sign(dx, w << (31 - WP_SD)));
+    h = flip_sign(q, w << (31 - WP_SH));
+    if (w & WP_HIST) {  // eq. BC:elasticity: the outgoing population of the previous call
+        g = (w & WP_HOR) ? a.H[hor][3 * x + hslot(hor, opp8(K))] : a.H[vert][3 * y + hslot(vert, opp8(K))];
+        h = T(0);
+    }
+    if constexpr (kind_fine(KIND)) {
+        if (w & WP_DATA) {
+            const int side = (w & WP_HOR) ? hor : vert;
+            if (a.prof[side]) {
+                const int n = (w & WP_HOR) ? a.nx : a.ny;
+                if (a.bc[side] == BC_NEUMANN) g += T(a.c0h * traction_term(a.prof[side], side, n, x, y, cx, cy));
+                else g += T(dirichlet_term(a.prof[side], side, n, x, y, cx, cy));
+            }
+        }
+    }
+}
+
+// Pair p after streaming: the small parts of S = g_first + g_second and A =
+// g_first - g_second.  (Their beta parts -- the beta sum, and the beta difference
+// minus a_p -- vanish exactly away from walls; at a wall the wall table has them.)
 template <typename T>
 struct PairOut {
-    T Ss, As;      // small parts
-    T bsx, bsy;    // beta sum (S)
-    T dbx, dby;    // beta difference minus a_p (A)
+    T Ss, As;
 };
 
-template <typename T, int P>
-__device__ __forceinline__ PairOut<T> pair_from(const PVal<T> &u, const PVal<T> &v);
-
-template <typename T, typename TC, int KIND, bool LO, int W, int P, bool WALL>
-__device__ __forceinline__ PairOut<T> pull_pair(const SweepArgs<T, TC> &a, const Rings<T, W, KIND, LO> &rg, int x, int y,
-                                                const int (&sl)[3], int c0, T tx, T ty, T tlx, T tly, bool perx, bool pery)
-{
-    const PVal<T> u = pull<T, TC, KIND, LO, W, pair_first(P), WALL>(a, rg, x, y, sl, c0, tx, ty, tlx, tly, perx, pery);
-    const PVal<T> v = pull<T, TC, KIND, LO, W, pair_second(P), WALL>(a, rg, x, y, sl, c0, tx, ty, tlx, tly, perx, pery);
-    return pair_from<T, P>(u, v);
-}
-
-template <typename T, int P>
-__device__ __forceinline__ PairOut<T> pair_from(const PVal<T> &u, const PVal<T> &v)
+template <typename T>
+__device__ __forceinline__ PairOut<T> pair_from(T ug, T uh, T vg, T vh)
 {
     PairOut<T> o;
-    o.Ss = (u.g + v.g) + (u.h + v.h);
-    o.As = (u.g - v.g) + (u.h - v.h);
-    o.bsx = u.bx + v.bx;
-    o.bsy = u.by + v.by;
-    o.dbx = (u.bx - v.bx) - T(pa_x(P));
-    o.dby = (u.by - v.by) - T(pa_y(P));
+    o.Ss = (ug + vg) + (uh + vh);
+    o.As = (ug - vg) + (uh - vh);
     return o;
 }
+template <typename T>
+__device__ __forceinline__ PairOut<T> pair_from(const PVal<T> &u, const PVal<T> &v)
+{
+    return pair_from(u.g, u.h, v.g, v.h);
+}
 
-template <typename T, typename TC, bool LO, int W, int KIND, int K>
-__device__ __forceinline__ void store_history(const SweepArgs<T, TC> &a, const Rings<T, W, KIND, LO> &rg, int side, int pos,
+template <typename T, bool LO, int K, typename A, typename RG>
+__device__ __forceinline__ void store_history(const A &a, const RG &rg, int side, int pos,
                                               int s0, int c0, T tx, T ty, T tlx, T tly)
 {
-    const PVal<T> o = post_at<T, LO, W, KIND, K>(rg, s0, c0, tx, ty, tlx, tly);
+    const PVal<T> o = post_at<T, LO, K>(rg, s0, c0, tx, ty, tlx, tly);
     a.H[side][3 * pos + hslot(side, K)] = (o.g + o.h) + (mul_rn(o.bx, tx + tlx) + mul_rn(o.by, ty + tly));
 }
 
@@ -635,35 +633,53 @@ __device__ __forceinline__ void residual_core(const OwnCell<T> &own, const PairO
 }
 
 // Residual d = m - m** of the cell (x, y) (small parts only, see the file
-// comment); own: the cell's own values.
-template <typename T, typename TC, int KIND, bool LO, int W, bool WALL>
-__device__ __forceinline__ void residual_cell(const SweepArgs<T, TC> &a, const Rings<T, W, KIND, LO> &rg, int x, int y,
-                                              const int (&sl)[3], int c0, bool perx, bool pery, const OwnCell<T> &own,
-                                              T (&d)[8])
+// comment); own: the cell's own values; E, G: a wall cell's table entry.
+template <typename T, int KIND, bool LO, bool WALL, typename A, typename RG>
+__device__ __forceinline__ void residual_cell(const A &a, const RG &rg, int x, int y, const int (&sl)[3], int c0,
+                                              const OwnCell<T> &own, T (&d)[8], const WallEntry<T> &E,
+                                              const WallGhost<T> &G)
 {
     const int s0 = sl[1];
-    const T(&gcur)[8] = own.g;
     const T tx = own.tx, ty = own.ty, tlx = own.tlx, tly = own.tly;
-#define BIOT_PAIR(P) pull_pair<T, TC, KIND, LO, W, P, WALL>(a, rg, x, y, sl, c0, tx, ty, tlx, tly, perx, pery)
-    const PairOut<T> P0 = BIOT_PAIR(0), P1 = BIOT_PAIR(1), P2 = BIOT_PAIR(2), P3 = BIOT_PAIR(3);
-#undef BIOT_PAIR
-    residual_core<T, KIND, LO>(own, P0, P1, P2, P3, d);
+    if constexpr (!WALL) {
+#define BIOT_POST(K) post_at<T, LO, K>(rg, sl[1 - ey8(K)], c0 - ex8(K), tx, ty, tlx, tly)
+        residual_core<T, KIND, LO>(own, pair_from(BIOT_POST(0), BIOT_POST(2)), pair_from(BIOT_POST(1), BIOT_POST(3)),
+                                   pair_from(BIOT_POST(4), BIOT_POST(6)), pair_from(BIOT_POST(5), BIOT_POST(7)), d);
+#undef BIOT_POST
+    } else {
+        T g[8], h[8];
+#define BIOT_PULL(K) wall_pull_at<T, KIND, LO, K>(a, rg, E.pull[K], x, y, sl, c0, tx, ty, tlx, tly, g[K], h[K])
+        BIOT_PULL(0);
+        BIOT_PULL(1);
+        BIOT_PULL(2);
+        BIOT_PULL(3);
+        BIOT_PULL(4);
+        BIOT_PULL(5);
+        BIOT_PULL(6);
+        BIOT_PULL(7);
+#undef BIOT_PULL
+        residual_core<T, KIND, LO>(own, pair_from(g[0], h[0], g[2], h[2]), pair_from(g[1], h[1], g[3], h[3]),
+                                   pair_from(g[4], h[4], g[6], h[6]), pair_from(g[5], h[5], g[7], h[7]), d);
+    }
     const T mxf = tx + tlx, myf = ty + tly;
     constexpr bool GH = kind_ghosts(KIND);
     if (WALL) {
         // beta terms of the wall pulls; products rounded on their own (mul_rn), so
         // that no contraction choice of the compiler makes kernel forms differ
-        d[0] -= mul_rn((P0.dbx + P2.dbx) - P3.dbx, mxf) + mul_rn((P0.dby + P2.dby) - P3.dby, myf);
-        d[1] -= mul_rn((P1.dbx + P2.dbx) + P3.dbx, mxf) + mul_rn((P1.dby + P2.dby) + P3.dby, myf);
-        d[5] -= mul_rn(P2.dbx - P3.dbx, mxf) + mul_rn(P2.dby - P3.dby, myf);
-        d[6] -= mul_rn(P2.dbx + P3.dbx, mxf) + mul_rn(P2.dby + P3.dby, myf);
-        d[2] -= mul_rn(P2.bsx - P3.bsx, mxf) + mul_rn(P2.bsy - P3.bsy, myf);
-        d[3] -= mul_rn((P0.bsx + P1.bsx) + T(2) * (P2.bsx + P3.bsx), mxf) +
-                mul_rn((P0.bsy + P1.bsy) + T(2) * (P2.bsy + P3.bsy), myf);
-        d[4] -= mul_rn(P0.bsx - P1.bsx, mxf) + mul_rn(P0.bsy - P1.bsy, myf);
-        d[7] -= mul_rn(P2.bsx + P3.bsx, mxf) + mul_rn(P2.bsy + P3.bsy, myf);
+        if (E.beta) {
+            d[0] -= mul_rn(E.bd[0][0], mxf) + mul_rn(E.bd[0][1], myf);
+            d[1] -= mul_rn(E.bd[1][0], mxf) + mul_rn(E.bd[1][1], myf);
+            d[2] -= mul_rn(E.bs[0][0], mxf) + mul_rn(E.bs[0][1], myf);
+            d[3] -= mul_rn(E.bs[1][0], mxf) + mul_rn(E.bs[1][1], myf);
+            d[4] -= mul_rn(E.bs[2][0], mxf) + mul_rn(E.bs[2][1], myf);
+            if constexpr (GH) {
+                d[5] -= mul_rn(G.b[0][0], mxf) + mul_rn(G.b[0][1], myf);
+                d[6] -= mul_rn(G.b[1][0], mxf) + mul_rn(G.b[1][1], myf);
+                d[7] -= mul_rn(G.b[2][0], mxf) + mul_rn(G.b[2][1], myf);
+            }
+        }
         // history of the fullway bounce-back: this call's outgoing populations
-#define BIOT_HIST(SIDE, POS, K) store_history<T, TC, LO, W, KIND, K>(a, rg, SIDE, POS, s0, c0, tx, ty, tlx, tly)
+#define BIOT_HIST(SIDE, POS, K) store_history<T, LO, K>(a, rg, SIDE, POS, s0, c0, tx, ty, tlx, tly)
         if (y == 0 && a.bc[SIDE_BOTTOM] == BC_DIRICHLET) { BIOT_HIST(SIDE_BOTTOM, x, 3); BIOT_HIST(SIDE_BOTTOM, x, 6); BIOT_HIST(SIDE_BOTTOM, x, 7); }
         if (y == a.ny - 1 && a.bc[SIDE_TOP] == BC_DIRICHLET) { BIOT_HIST(SIDE_TOP, x, 1); BIOT_HIST(SIDE_TOP, x, 4); BIOT_HIST(SIDE_TOP, x, 5); }
         if (x == 0 && a.bc[SIDE_LEFT] == BC_DIRICHLET) { BIOT_HIST(SIDE_LEFT, y, 2); BIOT_HIST(SIDE_LEFT, y, 5); BIOT_HIST(SIDE_LEFT, y, 6); }
@@ -820,8 +836,13 @@ __device__ __forceinline__ void sweep_strip(const SweepArgs<T, TC> &a, int bx, i
             if (writes[j]) {
                 const OwnCell<T> own = own_cell<T, W, KIND, LO>(rg, sb, c);
                 const T(&gcur)[8] = own.g;
-                if (!INT && (wall_col[j] || wall_row)) residual_cell<T, TC, KIND, LO, W, true>(a, rg, x, y, sl, c, perx, pery, own, d);
-                else residual_cell<T, TC, KIND, LO, W, false>(a, rg, x, y, sl, c, perx, pery, own, d);
+                const WallTable<T> &WT = wall_table<T>();
+                if (!INT && (wall_col[j] || wall_row)) {
+                    const int wi = wall_cell_index(a, x, y, perx, pery);
+                    residual_cell<T, KIND, LO, true>(a, rg, x, y, sl, c, own, d, WT.e[wi], WT.g[wi]);
+                } else {
+                    residual_cell<T, KIND, LO, false>(a, rg, x, y, sl, c, own, d, WT.e[0], WT.g[0]);
+                }
                 if (!RESTRICT) {
                     store_smoothed<T, TC, KIND, LO>(a, (size_t)y * nx + x, NP, own, d, gam);
                     if (a.resmax) {
@@ -950,7 +971,7 @@ __device__ __forceinline__ void sweep_strip_reg(const SweepArgs<T, TC> &a, int b
     auto collide = [&](const T (&R)[RV], T msS, T msN, int sm, int s, int sp, T &g1, T &g3, T &my) {
         T e[NE];
         extras(R, e);
-        const CollideOut<T> o = collide_math<T, TC, KIND, LO, NE>(
+        const CollideOut<T> o = collide_math<T, KIND, LO, NE>(
             a, R[0], R[1], R[2], R[3], R[4], e, MSR(s, t + 1), MSR(s, t - 1), msN, msS, MSR(sp, t + 1),
             MSR(sp, t - 1), MSR(sm, t + 1), MSR(sm, t - 1));
         PST(s, 0, t) = o.G[0];
@@ -1032,8 +1053,8 @@ __device__ __forceinline__ void sweep_strip_reg(const SweepArgs<T, TC> &a, int b
             const PVal<T> p5 = pval_from<T, LO, 5>(PST(sa, 3, t + 1), PST(sa, 6, t + 1), PST(sa, 7, t + 1), tx, ty, tlx, tly);
             const PVal<T> p6 = pval_from<T, LO, 6>(PST(sc, 4, t + 1), PST(sc, 6, t + 1), PST(sc, 7, t + 1), tx, ty, tlx, tly);
             const PVal<T> p7 = pval_from<T, LO, 7>(PST(sc, 5, t - 1), PST(sc, 6, t - 1), PST(sc, 7, t - 1), tx, ty, tlx, tly);
-            residual_core<T, KIND, LO>(own, pair_from<T, 0>(p0, p2), pair_from<T, 1>(p1, p3), pair_from<T, 2>(p4, p6),
-                                       pair_from<T, 3>(p5, p7), d);
+            residual_core<T, KIND, LO>(own, pair_from(p0, p2), pair_from(p1, p3), pair_from(p4, p6),
+                                       pair_from(p5, p7), d);
             d[5] = d[6] = d[7] = T(0);  // elided ghost moments
             if (!RESTRICT) {
                 store_smoothed<T, TC, KIND, LO>(a, (size_t)y * nx + x, NP, own, d, gam);
@@ -1183,6 +1204,18 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T, TC> &a, int bx, int
     const bool xin = perx || (x >= 0 && x < nx);
     const bool yin = pery || (y >= 0 && y < ny);
 
+    // A warp with a wall cell among its written cells takes the wall form for
+    // all of them: it then runs one form instead of both one after the other
+    // (the slowest warp sets a tile's time at its barriers).  For a cell away
+    // from the walls the wall form adds zero terms (exactly zero coefficients):
+    // the values are the same, up to the sign of an exact zero.  The cells' wall
+    // table entries are loaded together with the cells.
+    const bool writes = live && c >= 2 && c < W - 2 && rrow >= 2 && rrow < R - 2 && x < nx && y < ny;
+    const bool wall_cell = writes && ((!perx && (x == 0 || x == nx - 1)) || (!pery && (y == 0 || y == ny - 1)));
+    const bool wall = __any_sync(0xffffffffu, wall_cell);
+    const int wi = wall_cell ? wall_cell_index(a, x, y, perx, pery) : 0;
+    WallEntry<T> E;
+    if (wall) E = wall_table<T>().e[wi];
     if (live && (perx || x < nx + 2) && (pery || y < ny + 2)) {
         T pv[RV];
         fetch_cell<T, TC, KIND, LO, RV>(a, x, y, NP, perx, pery, pv);
@@ -1195,14 +1228,6 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T, TC> &a, int bx, int
 
     T rmax = T(0), gmax = T(0);
     double rsum = 0.0;
-    const bool writes = live && c >= 2 && c < W - 2 && rrow >= 2 && rrow < R - 2 && x < nx && y < ny;
-    // A warp with a wall cell among its written cells takes the wall form for
-    // all of them: it then runs one form instead of both one after the other
-    // (the slowest warp sets a tile's time at its barriers).  For a cell away
-    // from the walls the wall form adds zero terms (exactly zero coefficients):
-    // the values are the same, up to the sign of an exact zero.
-    const bool wall_cell = writes && ((!perx && (x == 0 || x == nx - 1)) || (!pery && (y == 0 || y == ny - 1)));
-    const bool wall = __any_sync(0xffffffffu, wall_cell);
     T d[8];
 #pragma unroll
     for (int k = 0; k < 8; k++) d[k] = T(0);
@@ -1210,8 +1235,8 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T, TC> &a, int bx, int
         const int sl[3] = {rrow - 1, rrow, rrow + 1};
         const OwnCell<T> own = own_cell<T, W, KIND, LO>(rg, rrow, c);
         const T(&gcur)[8] = own.g;
-        if (wall) residual_cell<T, TC, KIND, LO, W, true>(a, rg, x, y, sl, c, perx, pery, own, d);
-        else residual_cell<T, TC, KIND, LO, W, false>(a, rg, x, y, sl, c, perx, pery, own, d);
+        if (wall) residual_cell<T, KIND, LO, true>(a, rg, x, y, sl, c, own, d, E, wall_table<T>().g[wi]);
+        else residual_cell<T, KIND, LO, false>(a, rg, x, y, sl, c, own, d, E, wall_table<T>().g[0]);
         if (!RESTRICT) {
             store_smoothed<T, TC, KIND, LO>(a, (size_t)y * nx + x, NP, own, d, a.k_gam);
             if (a.resmax) {
