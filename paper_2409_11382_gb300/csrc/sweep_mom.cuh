@@ -465,14 +465,25 @@ __device__ __forceinline__ double flip_sign(double v, unsigned bit)
     return __hiloint2double(__double2hiint(v) ^ (int)(bit & 0x80000000u), __double2loint(v));
 }
 
-// The walls cell (x, y) touches, as an index of the wall table.
+// The walls cell (x, y) touches: bit 0 left, 1 right, 2 bottom, 3 top.
+template <typename A>
+__device__ __forceinline__ int wall_cell_class(const A &a, int x, int y, bool perx, bool pery)
+{
+    return (!perx && x == 0 ? 1 : 0) | (!perx && x == a.nx - 1 ? 2 : 0) | (!pery && y == 0 ? 4 : 0) |
+           (!pery && y == a.ny - 1 ? 8 : 0);
+}
+// A class as an index of the wall table.
+template <typename A>
+__device__ __forceinline__ int wall_class_index(const A &a, int c)
+{
+    auto kind = [&](int side) { return a.bc[side] == BC_DIRICHLET && a.hist_valid ? (int)WALL_DIR : a.bc[side]; };
+    return wall_index(c & 1 ? kind(SIDE_LEFT) : 0, c & 2 ? kind(SIDE_RIGHT) : 0, c & 4 ? kind(SIDE_BOTTOM) : 0,
+                      c & 8 ? kind(SIDE_TOP) : 0);
+}
 template <typename A>
 __device__ __forceinline__ int wall_cell_index(const A &a, int x, int y, bool perx, bool pery)
 {
-    auto kind = [&](int side) { return a.bc[side] == BC_DIRICHLET && a.hist_valid ? (int)WALL_DIR : a.bc[side]; };
-    const int eL = !perx && x == 0 ? kind(SIDE_LEFT) : 0, eR = !perx && x == a.nx - 1 ? kind(SIDE_RIGHT) : 0;
-    const int eB = !pery && y == 0 ? kind(SIDE_BOTTOM) : 0, eT = !pery && y == a.ny - 1 ? kind(SIDE_TOP) : 0;
-    return wall_index(eL, eR, eB, eT);
+    return wall_class_index(a, wall_cell_class(a, x, y, perx, pery));
 }
 
 // Population of direction K arriving at a wall cell (x, y) (ring column c0), as
@@ -751,6 +762,23 @@ __device__ __forceinline__ void sweep_strip(const SweepArgs<T, TC> &a, int bx, i
     const int x0 = bx * (W - 4), y0 = by * TY;
     const int y1 = min(y0 + TY, ny);
 
+    // the wall table's entries of this launch's walls, by class: a strip's rows
+    // stream through L1 and would evict them between two rows (read from global
+    // memory each row, the strips at the walls made the 4096^2 step 6 % slower)
+    constexpr bool GH = kind_ghosts(KIND);
+    __shared__ WallEntry<T> wall_e[INT ? 1 : 16];
+    __shared__ WallGhost<T> wall_g[INT || !GH ? 1 : 16];
+    if constexpr (!INT) {
+        constexpr int NW = sizeof(WallEntry<T>) / sizeof(unsigned), NG = sizeof(WallGhost<T>) / sizeof(unsigned);
+        for (int i = t; i < 16 * NW; i += NT)
+            reinterpret_cast<unsigned *>(wall_e)[i] =
+                reinterpret_cast<const unsigned *>(&wall_table<T>().e[wall_class_index(a, i / NW)])[i % NW];
+        if constexpr (GH)
+            for (int i = t; i < 16 * NG; i += NT)
+                reinterpret_cast<unsigned *>(wall_g)[i] =
+                    reinterpret_cast<const unsigned *>(&wall_table<T>().g[wall_class_index(a, i / NG)])[i % NG];
+    }
+
     // this thread's columns x[j] = x0 - 2 + c[j], ring columns c[j] = t + j NT
     int xj[CPT], cj[CPT];
     bool loads[CPT], collides[CPT], writes[CPT], wall_col[CPT];
@@ -836,12 +864,11 @@ __device__ __forceinline__ void sweep_strip(const SweepArgs<T, TC> &a, int bx, i
             if (writes[j]) {
                 const OwnCell<T> own = own_cell<T, W, KIND, LO>(rg, sb, c);
                 const T(&gcur)[8] = own.g;
-                const WallTable<T> &WT = wall_table<T>();
                 if (!INT && (wall_col[j] || wall_row)) {
-                    const int wi = wall_cell_index(a, x, y, perx, pery);
-                    residual_cell<T, KIND, LO, true>(a, rg, x, y, sl, c, own, d, WT.e[wi], WT.g[wi]);
+                    const int wc = wall_cell_class(a, x, y, perx, pery);
+                    residual_cell<T, KIND, LO, true>(a, rg, x, y, sl, c, own, d, wall_e[INT ? 0 : wc], wall_g[INT || !GH ? 0 : wc]);
                 } else {
-                    residual_cell<T, KIND, LO, false>(a, rg, x, y, sl, c, own, d, WT.e[0], WT.g[0]);
+                    residual_cell<T, KIND, LO, false>(a, rg, x, y, sl, c, own, d, wall_e[0], wall_g[0]);
                 }
                 if (!RESTRICT) {
                     store_smoothed<T, TC, KIND, LO>(a, (size_t)y * nx + x, NP, own, d, gam);
@@ -1167,7 +1194,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 896 / (NT * CPT) : 1) k_s
 // global round trip and one pass of arithmetic per launch instead of a walk
 // down a strip.  Rows of the tile are the ring slots of the strip kernel, so the
 // same collision, pull and residual code runs.  Restriction sums 2 x 2 blocks
-// of the tile (TX, TY even) through shared memory.
+// of the tile (TX, TY even) through shared memory.  Only rows ylo .. yhi-1 (even
+// bounds) are written.
 // ---------------------------------------------------------------------------
 template <int TX, int TY>
 struct TileShape {
@@ -1183,7 +1211,7 @@ constexpr size_t tile_smem_bytes()
 
 template <typename T, typename TC, int TX, int TY, int KIND, bool LO, bool RESTRICT>
 __device__ __forceinline__ void tile_body(const SweepArgs<T, TC> &a, int bx, int by, unsigned char *smem_raw,
-                                          double (&red)[3][TileShape<TX, TY>::NT / 32])
+                                          double (&red)[3][TileShape<TX, TY>::NT / 32], int ylo = 0, int yhi = 0x7fffffff)
 {
     using L = RingLayout<KIND, LO>;
     using S = TileShape<TX, TY>;
@@ -1210,7 +1238,7 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T, TC> &a, int bx, int
     // from the walls the wall form adds zero terms (exactly zero coefficients):
     // the values are the same, up to the sign of an exact zero.  The cells' wall
     // table entries are loaded together with the cells.
-    const bool writes = live && c >= 2 && c < W - 2 && rrow >= 2 && rrow < R - 2 && x < nx && y < ny;
+    const bool writes = live && c >= 2 && c < W - 2 && rrow >= 2 && rrow < R - 2 && x < nx && y < ny && y >= ylo && y < yhi;
     const bool wall_cell = writes && ((!perx && (x == 0 || x == nx - 1)) || (!pery && (y == 0 || y == ny - 1)));
     const bool wall = __any_sync(0xffffffffu, wall_cell);
     const int wi = wall_cell ? wall_cell_index(a, x, y, perx, pery) : 0;
@@ -1256,7 +1284,7 @@ __device__ __forceinline__ void tile_body(const SweepArgs<T, TC> &a, int bx, int
         if (tid < (TX / 2) * (TY / 2)) {
             const int bx = tid % (TX / 2), by = tid / (TX / 2);
             const int xc = x0 / 2 + bx, yc = y0 / 2 + by;
-            if (2 * xc < nx && 2 * yc < ny) {
+            if (2 * xc < nx && 2 * yc < ny && 2 * yc >= ylo && 2 * yc < yhi) {
                 const size_t NPc = NP >> 2;
                 const size_t cidx = (size_t)yc * (nx >> 1) + xc;
                 const int i0 = (2 * by) * TX + 2 * bx;
