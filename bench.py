@@ -517,7 +517,7 @@ def run_ours(args):
                    "precision": precision_label(params, fp64),
                    "l2": f"state ({st['device_bytes'] / 1e9:.1f} GB) larger than L2; no flush needed",
                    "parallelism": f"replicas{world}",
-                   "coarse_sweeps": "cluster segments" if args.segments else "separate graph-launched kernels",
+                   "coarse_sweeps": "cluster launches, BIOT_OPT_SEGMENTS" if args.segments else "cluster launches below 64^2 (batch: 16^2)",
                    "autotuned_strip_rows": tuned},
         "roofline": roofline,
         "cpu_baseline": cpu_base,
@@ -685,7 +685,7 @@ def run_batched(args):
                        "cells_total": cells, "ne_fixed": 3, "K": 4,
                        "l2": "state of all instances larger than L2; no flush needed",
                        "parallelism": f"replicas{world}",
-                       "coarse_sweeps": "cluster segments" if args.segments else "separate graph-launched kernels",
+                       "coarse_sweeps": "cluster launches, BIOT_OPT_SEGMENTS" if args.segments else "cluster launches below 64^2 (batch: 16^2)",
                        "launches_per_step": st["launches_per_step"]},
             "e2e": {"value": cells * e2e_steps / e2e / 1e6, "unit": "MLUPS",
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h // e2e_steps,
@@ -813,7 +813,7 @@ def main():
     ap.add_argument("--cold", choices=["auto", "fp64", "fp32"], default="auto",
                     help="single, FP32 path: the solve at t = 0 on an FP64 copy (auto: from 2048^2 cells)")
     ap.add_argument("--segments", action="store_true",
-                    help="the sweeps of the small coarse levels as cluster segments (BIOT_OPT_SEGMENTS)")
+                    help="more of the small coarse levels in one cluster launch (BIOT_OPT_SEGMENTS)")
     ap.add_argument("--requests", type=int, default=200, help="served: number of requests")
     ap.add_argument("--mean-service", type=float, default=0.05, help="served: assumed mean service time (s)")
     ap.add_argument("--budget-gb", type=float, default=16.0, help="served: device-memory budget")

@@ -89,14 +89,13 @@ extern "C" {
 #define BIOT_OPT_COARSE_LO_ALL    8   /* double-float first moments on the FP32 coarse levels
                                          in every solve (default: in an FP32 solve at t = 0) */
 #define BIOT_OPT_COARSE_LO_OFF   16   /* ... in no solve */
-#define BIOT_OPT_SEGMENTS        32   /* a launch choice, honoured in every precision: the
-                                         sweeps of the small coarse levels of a V-cycle (at most 16
-                                         tiles each) as one thread-block-cluster launch per run of
-                                         sweeps of one storage type (one cluster per instance in a
-                                         batch) instead of one graph-launched kernel per sweep.
-                                         Results are bitwise the same; on GB300 it is measured
-                                         slower (graph launches cost about what the cluster
-                                         barriers cost), so it is off by default */
+#define BIOT_OPT_SEGMENTS        32   /* a launch choice, honoured in every precision.  By default
+                                         the coarse-grid correction below a small level (64^2 cells;
+                                         16^2 in a batch) is one thread-block-cluster launch that keeps
+                                         its levels in shared memory, one cluster per instance.  With
+                                         this flag that launch starts at levels of up to four times the
+                                         cells as far as they fit, and the solve at t = 0 takes it too:
+                                         fewer launches, bitwise the same results */
 
 /* ---- boundary condition types (§3.6) --------------------------------------- */
 #define BIOT_PERIODIC  0  /* wrap-around streaming; must be set on both opposite sides

@@ -30,7 +30,9 @@ UNITS = {
     "kernels_fp64.cu": ["--fmad=false"],
     "kernels_fp32.cu": [],
     "kernels_fp32c.cu": [],
-    "kernels_seg32.cu": [],
+    "kernels_batch32.cu": [],
+    "kernels_batch32c.cu": [],
+    "kernels_resident.cu": ["--fmad=false"],
 }
 
 

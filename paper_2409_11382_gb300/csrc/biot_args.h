@@ -76,7 +76,7 @@ struct SweepItem {
 
 // Storage kind of a sweep launch (bit flags).
 enum { SWEEP_V_COARSE = 1, SWEEP_V_LO = 2, SWEEP_V_RESTRICT = 4, SWEEP_V_NOGHOST = 8, SWEEP_V_TILE = 16,
-       SWEEP_V_DEV16 = 32, SWEEP_V_DEVBF16 = 64, SWEEP_V_SEGMENT = 128 };
+       SWEEP_V_DEV16 = 32, SWEEP_V_DEVBF16 = 64, SWEEP_V_RESIDENT = 128 };
 // Tile sweeps: levels of at most SWEEP_TILE_CELLS cells (single instance); tile
 // shape per storage type.  The fused flow step works on FLOW_TILE_X x FLOW_TILE_Y tiles.
 constexpr long SWEEP_TILE_CELLS = 256L * 256L;
@@ -183,13 +183,6 @@ struct StopArgs {
 cudaError_t launch_stop_test(const StopArgs &a, cudaStream_t s);
 
 template <typename T, typename TC> cudaError_t launch_sweep_mom(const SweepArgs<T, TC> &a, cudaStream_t s);
-// n consecutive smoothing sweeps of one small FP64 level (at most
-// SWEEP_CHAIN_MAX x SWEEP_CHAIN_MAX cells) in one launch: sweep k reads the
-// output of sweep k-1 (ping-pong between a.g and a.gout), only the first
-// sweep may start from zero (a.zero_init), the bounce-back history is valid
-// after it.  The result lies in a.g for even n and in a.gout for odd n.
-constexpr int SWEEP_CHAIN_MAX = 8;
-template <typename T, typename TC> cudaError_t launch_sweep_chain(const SweepArgs<T, TC> &a, int n, cudaStream_t s);
 // The jobs of one batched sweep launch, passed as a kernel parameter -- so that,
 // as in a single-instance launch, the arguments sit in constant memory rather
 // than in shared memory and registers.  Job j owns the work items
@@ -208,64 +201,53 @@ struct BatchParams {
 // `variant` (SWEEP_V_* flags).
 template <typename T, typename TC>
 cudaError_t launch_sweep_batch(int variant, const BatchParams<T, TC> &P, cudaStream_t s);
-// Segment of a V-cycle: consecutive sweeps of small coarse levels of one
-// storage family (T = float: levels of tkind float/float and float/double;
-// T = double: double/double) run by one thread-block cluster in one launch, a
-// cluster barrier between the sweeps.  A program is the sweeps of one
-// instance's segment; one launch runs one program per cluster (one cluster per
-// instance of a batch).  Each level of a program has one record: its sweep
-// arguments with the parts that change from sweep to sweep (iterate buffers,
-// prolongation source, restriction target, flags) taken from the sweep's job
-// word.  Everything is a kernel parameter, so a launch captured in a graph
-// needs no device table.
-struct SegLevel {
-    union {
-        SweepArgs<double, double> dd;
-        SweepArgs<float, double> fd;
-        SweepArgs<float, float> ff;
-    } a;                  // base arguments; g, gout, gc, rc, zero_init, hist_valid, mode set per sweep
-    const void *buf[2];   // the level's two iterate buffers
-    const void *cbuf[2];  // the next coarser level's two iterate buffers (prolongation source)
-    void *crc;            // the next coarser level's residual right-hand side (restriction target)
-    int tkind;            // 0: double/double, 1: float/double, 2: float/float
-    int pad;
+// Resident cycle (sweep_resident.cuh): one multigrid cycle on the correction
+// problem of a coarse level and the levels below it, run by one thread-block
+// cluster with the levels in shared memory.  lev[0] is the top level; a level's
+// rows are dealt out in runs of rpc to the first nranks CTAs of the cluster.
+// Offsets are bytes into each CTA's dynamic shared memory.
+constexpr int RES_MAX_LEVELS = 8;     // levels of one program
+constexpr int RES_MAX_OPS = 160;      // operations of one program
+constexpr int RES_MAX_PROGS = 46;     // programs (instances) of one launch: a parameter block below 32 KB
+constexpr int RES_NT = 512;           // threads of a CTA
+constexpr int RES_CLUSTER_MAX = 16;   // CTAs of a cluster (above 8: the non-portable size)
+constexpr int RES_SMEM_MAX = 220 * 1024;
+// Operations: K smoothing sweeps of a level; residual and restriction from a
+// level to the next coarser one, whose iterate becomes zero; prolongation of that
+// level's iterate into this one's.
+enum { RES_OP_LEVEL = 15, RES_OP_SMOOTH = 0, RES_OP_DOWN = 16, RES_OP_UP = 32 };
+struct ResLevel {
+    int nx, ny, rpc, nranks;
+    int K;                   // smoothing sweeps of one RES_OP_SMOOTH
+    int fp64;
+    unsigned inv;            // ceil(2^20 / rpc): y / rpc = y inv >> 20 for y < 4096
+    unsigned m, x, H, map;   // iterate, right-hand side, bounce-back history, cell list
+    unsigned cvt;            // FP64 level below an FP32 one: its iterate rounded to FP32
 };
-// Job word of one sweep: bits 0-3 the level record (relative to the program's
-// first), bit 4 restriction, bit 5 the parity of the input buffer, bit 6 zero
-// iterate, bit 7 prolongation (add the coarser level's buffer cbuf[bit 8]), bit 9
-// history valid.
-enum { SEGJ_LEVEL = 15, SEGJ_RESTRICT = 16, SEGJ_CUR = 32, SEGJ_ZERO = 64, SEGJ_PROL = 128, SEGJ_CCUR = 256,
-       SEGJ_HIST = 512 };
-// The arguments of job word w from its level record: the host builds the
-// words with this function's inverse and checks that it reproduces every sweep.
-template <typename T, typename TC>
-__host__ __device__ inline void seg_patch(SweepArgs<T, TC> &a, const SegLevel &L, unsigned w)
-{
-    const int cur = (w & SEGJ_CUR) ? 1 : 0;
-    const bool rs = (w & SEGJ_RESTRICT) != 0;
-    a.g = static_cast<const T *>(L.buf[cur]);
-    a.gout = rs ? nullptr : const_cast<T *>(static_cast<const T *>(L.buf[1 - cur]));
-    a.gc = (w & SEGJ_PROL) ? static_cast<const TC *>(L.cbuf[(w & SEGJ_CCUR) ? 1 : 0]) : nullptr;
-    a.rc = rs ? static_cast<TC *>(L.crc) : nullptr;
-    a.zero_init = (w & SEGJ_ZERO) ? 1 : 0;
-    a.hist_valid = (w & SEGJ_HIST) ? 1 : 0;
-    a.mode = rs ? SWEEP_RESTRICT : SWEEP_SMOOTH;
-}
-constexpr int SEG_MAX_PROGS = 32, SEG_MAX_LEVELS = 60, SEG_MAX_JOBS = 1200;
-constexpr int SEG_CLUSTER = 8;    // CTAs per cluster (the portable maximum)
-constexpr int SEG_MAX_TILES = 2 * SEG_CLUSTER;  // tiles of a level in a segment: at most 2 per CTA
-struct SegParams {
-    int nprog;
-    int ghosts;                   // 1: the ghost moments are loaded and stored (tolerance mode)
-    int lev0[SEG_MAX_PROGS + 1];  // program p: level records lev0[p] .. lev0[p+1]-1
-    int job0[SEG_MAX_PROGS + 1];  // program p: jobs job0[p] .. job0[p+1]-1
-    SegLevel lev[SEG_MAX_LEVELS];
-    unsigned job[SEG_MAX_JOBS];
+struct ResProg {
+    int nlev, nops;
+    int bc[4];
+    int zero;                // 1: the top level starts from a zero iterate
+    int hist_valid;          // 1: its bounce-back history is loaded (H)
+    int keep_hist;           // 1: it is stored again at the end
+    unsigned ms, post, dres; // work areas, shared by the levels
+    const void *r;           // right-hand side of the top level (5 planes)
+    void *g;                 // its iterate
+    void *H[4];
+    float kf[5];             // k_fs, k_hs, k_hd, k_h22, k_gam of SweepArgs in FP32 and FP64
+    double kd[5];
+    ResLevel lev[RES_MAX_LEVELS];
+    unsigned char ops[RES_MAX_OPS];
 };
-// One launch of P.nprog clusters of cs CTAs (1 <= cs <= SEG_CLUSTER); T selects
-// the storage family of every job.
-template <typename T>
-cudaError_t launch_sweep_segment(const SegParams &P, int cs, cudaStream_t s);
+struct ResParams {
+    int nprog, cs, ghosts;   // ghosts: 1 keeps the ghost moments (tolerance mode)
+    ResProg p[RES_MAX_PROGS];
+};
+static_assert(sizeof(ResParams) <= 32764, "the limit of a kernel's parameters");
+// P.nprog clusters of P.cs CTAs with smem bytes of dynamic shared memory each.
+cudaError_t launch_resident(const ResParams &P, size_t smem, cudaStream_t s);
+// CTAs of the largest cluster the device runs (RES_CLUSTER_MAX, or the portable 8).
+int resident_max_cluster();
 // Resident CTAs of a batched sweep launch (sweep_slots) and of a
 // single-instance strip launch (sweep_strip_slots) of this kind on the current
 // device, and the strip geometry of the two strip kernels (output columns per

@@ -40,15 +40,14 @@ struct SweepJob {
     SweepArgs<double, double> dd;
     SweepArgs<float, double> fd;
     SweepArgs<float, float> ff;
-    int seg = -1;  // SWEEP_V_SEGMENT: index of its program among the instance's recorded ones
+    int res = -1;  // SWEEP_V_RESIDENT: index of its program among the instance's recorded ones
 };
-// The program of one segment of a V-cycle (sweep_segment.cuh): the records of
-// its levels and one job word per sweep.
-struct SegProg {
-    int fam = 1;  // storage family: 0 double (tkind 0), 1 float (tkinds 1 and 2)
-    int cs = 1;   // CTAs per cluster: the most tiles of any of its levels, at most SEG_CLUSTER
-    std::vector<SegLevel> lev;
-    std::vector<unsigned> job;
+// The launch of one resident V-cycle (sweep_resident.cuh): its program and the
+// shared memory and cluster size it needs.
+struct ResLaunch {
+    ResProg prog;
+    size_t smem = 0;
+    int cs = 1;
 };
 // A flow step prepared for a batched launch.
 struct FlowRec {
@@ -258,9 +257,8 @@ struct biot_ctx {
     // record mode (batched execution): sweeps are appended here instead of launched
     std::vector<biot::SweepJob> *rec = nullptr;
     std::vector<biot::FlowRec> *frec = nullptr;  // record mode: flow steps appended here
-    std::vector<biot::SegProg> *segrec = nullptr;  // record mode: programs of the recorded segments
-    bool in_seg = false;  // recording the sweeps of a segment (seg_vcycle)
-    bool batched = false; // an instance of a batch (its steps are recorded and merged)
+    std::vector<biot::ResLaunch> *resrec = nullptr;  // record mode: the recorded resident V-cycles
+    bool batched = false;  // an instance of a batch
     // Allocation source of a server's instance: the server's stream-ordered
     // pool, so that freeing the instance synchronises only its own stream
     // (cudaFree would wait for every resident instance); its two pinned host
@@ -452,7 +450,7 @@ bool level_lo(const biot_ctx *h, int l, bool cold)
 }
 
 template <typename T, typename TC>
-int sweep_typed(biot_ctx *h, int l, int mode, bool zero_init, bool prolong, bool want_res, int chain)
+int sweep_typed(biot_ctx *h, int l, int mode, bool zero_init, bool prolong, bool want_res)
 {
     Level &Lv = h->lv[l];
     const bool fine = (l == h->L - 1);
@@ -523,225 +521,201 @@ int sweep_typed(biot_ctx *h, int l, int mode, bool zero_init, bool prolong, bool
         }
         CUDA_TRY(cudaEventRecord(h->ev[h->ev_used], h->stream));
     }
-    if (chain > 1) CUDA_TRY((launch_sweep_chain<T, TC>(a, chain, h->stream)));
-    else CUDA_TRY((launch_sweep_mom<T, TC>(a, h->stream)));
+    CUDA_TRY((launch_sweep_mom<T, TC>(a, h->stream)));
     if (timed) {
         CUDA_TRY(cudaEventRecord(h->ev[h->ev_used + 1], h->stream));
         h->ev_used += 2;
     }
     h->launches++;
     Lv.hist_valid = 1;
-    if (mode == SWEEP_SMOOTH && (chain <= 1 || (chain & 1))) Lv.cur ^= 1;
+    if (mode == SWEEP_SMOOTH) Lv.cur ^= 1;
     return BIOT_OK;
 }
 
-// chain > 1: that many smoothing sweeps of a small FP64 level in one launch.
-int sweep(biot_ctx *h, int l, int mode, bool zero_init, bool prolong, bool want_res, int chain = 1)
+int sweep(biot_ctx *h, int l, int mode, bool zero_init, bool prolong, bool want_res)
 {
     const bool t64 = h->lv[l].fp64;
     const bool c64 = (l > 0) ? h->lv[l - 1].fp64 : t64;
-    if (t64) return sweep_typed<double, double>(h, l, mode, zero_init, prolong, want_res, chain);
-    if (c64) return sweep_typed<float, double>(h, l, mode, zero_init, prolong, want_res, chain);
-    return sweep_typed<float, float>(h, l, mode, zero_init, prolong, want_res, chain);
+    if (t64) return sweep_typed<double, double>(h, l, mode, zero_init, prolong, want_res);
+    if (c64) return sweep_typed<float, double>(h, l, mode, zero_init, prolong, want_res);
+    return sweep_typed<float, float>(h, l, mode, zero_init, prolong, want_res);
 }
 
 // ---------------------------------------------------------------------------
-// Segments (BIOT_OPT_SEGMENTS).  The sweeps of the small coarse levels of a
-// V-cycle -- every level from the segment's start level down to the coarsest,
-// each of at most SEG_MAX_TILES tiles -- are recorded instead of launched, split
-// into runs of one storage family, and each run becomes one cluster launch of
-// k_sweep_segment (one cluster per instance).  Per-cell code and arguments are
-// those of the separate tile launches, so results are bitwise the same.  A
-// sweep inside a cluster costs what a graph-launched tile sweep costs (the
-// cluster barrier takes the place of the launch gap), and a 64^2 level's 16
-// tiles fall two to a CTA: measured slower than separate launches on GB300,
-// hence not the default.
+// Resident V-cycles (sweep_resident.cuh): the coarse-grid correction from a small
+// level down as one cluster launch.
 // ---------------------------------------------------------------------------
-int seg_tiles_of(const biot_ctx *h, int l)
+// Cells of a level that one CTA of the cluster takes before the next CTA gets
+// rows.  FP32 levels are latency-bound and a block barrier is cheaper than a
+// cluster barrier (128, 256 and 512 cells: 0.397, 0.383 and 0.394 ms per 64^2
+// step).  FP64 levels are bound by the FP64 instructions of an SM, so they spread
+// (16, 32 and 64 cells: 0.346, 0.348 and 0.371 ms); in a batch the SMs are taken
+// and the barriers are not worth it (16 and 64 cells: 6.74 and 6.63 ms per step of
+// the 64-instance workload).
+int res_min_cells(const biot_ctx *h, bool fp64) { return !fp64 ? 256 : h->batched ? 64 : 16; }
+
+// The largest level of a resident cycle, in cells.  Single instance: up to what
+// 16 CTAs hold, 64^2 in FP32 (against 32^2: 0.457 and 0.469 ms per 128^2 step,
+// 0.528 and 0.554 ms at 256^2, 1.62 and 1.66 ms at 1024^2) and 2048 cells in FP64
+// (against 1024: 0.600 and 0.686 ms per 64^2 FP64 step); with an FP32 coarsest
+// level 32^2, where 64^2 gains 1 % (0.793 and 0.801 ms at 512^2).  A batch's phase
+// launches fill the GPU, and a cluster holds SMs that they would use: 16^2 (6.63
+// ms per step of the 64-instance workload, 32^2: 6.77, 64^2: 7.75).
+long res_max_cells(const biot_ctx *h, bool fp64)
 {
-    int tx, ty;
-    sweep_tile_shape(h->lv[l].fp64, &tx, &ty);
-    return ((h->lv[l].nx + tx - 1) / tx) * ((h->lv[l].ny + ty - 1) / ty);
+    if (h->batched) return 256;
+    return fp64 ? 2048 : h->lv[0].fp64 ? 4096 : 1024;
 }
 
-// The level where a V-cycle's segment starts (-1: none): the finest coarse
-// level such that it and every coarser level have at most SEG_MAX_TILES tiles
-// and no double-float first moments (which the tile form of a segment does not
-// take).  cold: for the solve at t = 0.  With BIOT_OPT_SEGMENTS; without it,
-// only an instance of a batch has one, and only its FP64 coarsest level: the
-// 2K sweeps that a single instance runs as one chained launch.
-int seg_start(const biot_ctx *h, bool cold)
+// Threads that the fullest CTA of a level needs (level_sweeps): four lanes per cell
+// in FP64; in FP32 one per cell away from the walls, in whole warps, and four per
+// wall cell.
+int res_threads(bool fp64, int nx, int ny, int rpc)
 {
-    if (!(h->P.options & BIOT_OPT_SEGMENTS))
-        return (h->batched && h->L > 1 && h->lv[0].fp64 && seg_tiles_of(h, 0) <= SEG_MAX_TILES) ? 0 : -1;
+    int most = 0;
+    for (int r0 = 0; r0 < ny; r0 += rpc) {
+        const int r1 = std::min(r0 + rpc, ny);
+        const int ri = std::max(0, std::min(r1, ny - 1) - std::max(r0, 1)), inner = ri * std::max(0, nx - 2);
+        const int cells = (r1 - r0) * nx;
+        const int n = fp64 ? 4 * cells : ((inner + 31) & ~31) + 4 * (cells - inner);
+        most = std::max(most, (n + 31) & ~31);
+    }
+    return most;
+}
+
+// The operations of one cycle from program level l down, mirroring vcycle();
+// false when the program is full.
+bool res_ops(ResProg &P, int l, int kind)
+{
+    auto put = [&](int op) {
+        if (P.nops >= RES_MAX_OPS) return false;
+        P.ops[P.nops++] = (unsigned char)(op | l);
+        return true;
+    };
+    if (!put(RES_OP_SMOOTH)) return false;
+    if (l + 1 < P.nlev) {
+        if (!put(RES_OP_DOWN) || !res_ops(P, l + 1, kind)) return false;
+        if (kind != BIOT_CYCLE_V && !res_ops(P, l + 1, kind == BIOT_CYCLE_W ? BIOT_CYCLE_W : BIOT_CYCLE_V)) return false;
+        if (!put(RES_OP_UP)) return false;
+    }
+    return put(RES_OP_SMOOTH);
+}
+
+// Program and shared-memory plan of the cycle from level s down (no launch
+// addresses); false when it does not fit one cluster or one program.
+bool res_plan(const biot_ctx *h, int s, int kind, ResLaunch &R)
+{
+    ResProg &P = R.prog;
+    std::memset(&P, 0, sizeof(P));
+    if (s + 1 > RES_MAX_LEVELS) return false;
+    P.nlev = s + 1;
+    if (!res_ops(P, 0, kind)) return false;
+    for (int i = 0; i < 4; i++) P.bc[i] = h->bc_eta[i];
+    const int nm = h->P.ne_fixed > 0 ? 5 : 8, max_cs = resident_max_cluster();
+    size_t off = 0, ms = 0, post = 0, dres = 0;
+    auto take = [&](size_t bytes) {
+        const size_t o = off;
+        off += (bytes + 15) & ~(size_t)15;
+        return (unsigned)o;
+    };
+    R.cs = 1;
+    for (int l = s; l >= 0; l--) {
+        const Level &Lv = h->lv[l];
+        ResLevel &L = P.lev[s - l];
+        if (Lv.nx > 4095 || Lv.ny > 4095) return false;
+        const long cells = (long)Lv.nx * Lv.ny;
+        int want = (int)std::min<long>((cells + res_min_cells(h, Lv.fp64) - 1) / res_min_cells(h, Lv.fp64), max_cs);
+        while (want < max_cs && res_threads(Lv.fp64, Lv.nx, Lv.ny, (Lv.ny + want - 1) / want) > RES_NT) want++;
+        L.nx = Lv.nx;
+        L.ny = Lv.ny;
+        L.rpc = (Lv.ny + want - 1) / want;
+        L.nranks = (Lv.ny + L.rpc - 1) / L.rpc;
+        L.K = sweeps_of(&h->P, l);
+        L.fp64 = Lv.fp64;
+        R.cs = std::max(R.cs, L.nranks);
+        const size_t es = Lv.fp64 ? 8 : 4, cap = (size_t)L.rpc * L.nx, pad = (size_t)(L.rpc + 2) * L.nx;
+        if (L.rpc > 255 || res_threads(Lv.fp64, L.nx, L.ny, L.rpc) > RES_NT) return false;
+        L.inv = ((1u << 20) + L.rpc - 1) / L.rpc;
+        L.m = take(nm * cap * es);
+        L.x = take(5 * cap * es);
+        L.H = take(6 * (size_t)(L.nx + L.rpc) * es);
+        L.map = take(cap * sizeof(unsigned));
+        if (Lv.fp64 && l < s && !h->lv[l + 1].fp64) L.cvt = take(nm * cap * sizeof(float));
+        ms = std::max(ms, pad * es);
+        post = std::max(post, 10 * pad * es);
+        dres = std::max(dres, 5 * cap * es);
+    }
+    P.ms = take(ms);
+    P.post = take(post);
+    P.dres = take(dres);
+    R.smem = off;
+    return off <= (size_t)RES_SMEM_MAX;
+}
+
+// The finest level whose coarse-grid correction runs as one resident launch (-1:
+// none): every level down from it is within the bound and fits one cluster, and
+// none has double-float first moments (which the resident form does not take).
+// The solve at t = 0 runs once per instance and has them on its FP32 levels, so it
+// keeps one launch per sweep.  BIOT_OPT_SEGMENTS: levels of up to four times the
+// cells, and at t = 0 too.
+int res_start(const biot_ctx *h, bool cold, int kind = BIOT_CYCLE_V)
+{
+    const bool more = (h->P.options & BIOT_OPT_SEGMENTS) != 0;
+    if (cold && !more) return -1;
     int s = -1;
+    ResLaunch R;
     for (int l = 0; l < h->L - 1; l++) {
-        if (level_lo(h, l, cold) || seg_tiles_of(h, l) > SEG_MAX_TILES) break;
+        const long cells = (long)h->lv[l].nx * h->lv[l].ny;
+        const long bound = res_max_cells(h, h->lv[l].fp64);
+        if (level_lo(h, l, cold) || cells > (more ? 4 * bound : bound) || !res_plan(h, l, kind, R)) break;
         s = l;
     }
     return s;
 }
 
-template <typename X>
-bool seg_eq(const X &a, const X &b) { return std::memcmp(&a, &b, sizeof(X)) == 0; }
-
-// Field by field (padding aside): are two sweeps' arguments the same?  The
-// strip height `rows` is not compared: tile sweeps do not read it.
-template <typename T, typename TC>
-bool seg_same_args(const SweepArgs<T, TC> &a, const SweepArgs<T, TC> &b)
+// One cycle from level s down on level s's right-hand side, from a zero iterate
+// or the stored one; the result lands in the level's current buffer.  In record
+// mode (a batch) the program is recorded instead of launched.
+int res_cycle(biot_ctx *h, int s, bool zero_start, int kind)
 {
-    bool ok = a.nx == b.nx && a.ny == b.ny && a.g == b.g && a.gout == b.gout && a.glo == b.glo &&
-              a.glo_out == b.glo_out && a.r == b.r && a.Ft == b.Ft && a.gc == b.gc && a.rc == b.rc &&
-              a.hist_valid == b.hist_valid && a.zero_init == b.zero_init && a.mode == b.mode &&
-              seg_eq(a.gamma, b.gamma) && seg_eq(a.om_s, b.om_s) && seg_eq(a.om_d, b.om_d) && seg_eq(a.lm, b.lm) &&
-              seg_eq(a.coef_fstar, b.coef_fstar) && seg_eq(a.c0h, b.c0h) && a.resmax == b.resmax &&
-              a.ghosts == b.ghosts && seg_eq(a.k_fs, b.k_fs) && seg_eq(a.k_hs, b.k_hs) && seg_eq(a.k_hd, b.k_hd) &&
-              seg_eq(a.k_h22, b.k_h22) && seg_eq(a.k_gam, b.k_gam) && a.dev == b.dev && a.gd == b.gd &&
-              a.gd_out == b.gd_out && seg_eq(a.dsc, b.dsc) && seg_eq(a.dinv, b.dinv) && a.dev_full == b.dev_full;
-    for (int i = 0; i < 4; i++) ok = ok && a.H[i] == b.H[i] && a.prof[i] == b.prof[i] && a.bc[i] == b.bc[i];
-    return ok;
-}
-
-// Job word of one recorded sweep of level l (level record rel of the program),
-// checked to reproduce the sweep's arguments through seg_patch.
-template <typename T, typename TC>
-int seg_word(const biot_ctx *h, const SweepArgs<T, TC> &a, int l, const SegLevel &L, int rel, unsigned *out)
-{
-    const Level &Lv = h->lv[l];
-    unsigned w = (unsigned)rel;
-    if (a.mode == SWEEP_RESTRICT) w |= SEGJ_RESTRICT;
-    if (a.g == Lv.g[1]) w |= SEGJ_CUR;
-    if (a.zero_init) w |= SEGJ_ZERO;
-    if (a.gc) {
-        w |= SEGJ_PROL;
-        if (l > 0 && (const void *)a.gc == h->lv[l - 1].g[1]) w |= SEGJ_CCUR;
+    ResLaunch R;
+    if (!res_plan(h, s, kind, R)) return fail(BIOT_ERR_CUDA, "resident cycle does not fit one cluster");
+    ResProg &P = R.prog;
+    Level &Lv = h->lv[s];
+    P.zero = zero_start ? 1 : 0;
+    P.hist_valid = Lv.hist_valid;
+    P.keep_hist = kind != BIOT_CYCLE_V;  // a second cycle from this level may follow
+    P.r = Lv.r;
+    P.g = Lv.g[Lv.cur];
+    for (int i = 0; i < 4; i++) P.H[i] = Lv.H[i];
+    // the coefficients of SweepArgs, evaluated as sweep_typed does
+    const double k22 = -1.0 / (12.0 * h->lm + 4.0), cf = 0.5 * h->P.alpha * h->P.alpha * h->P.r_coupling;
+    const double k[5] = {cf * (-1.5 / (3.0 * h->lm + 1.0)), 0.25 * (1.0 - h->om_s) - 0.5 * k22, 0.25 * (1.0 - h->om_d),
+                         0.25 * k22, h->P.gamma};
+    for (int i = 0; i < 5; i++) {
+        P.kd[i] = k[i];
+        P.kf[i] = (float)k[i];
     }
-    if (a.hist_valid) w |= SEGJ_HIST;
-    SweepArgs<T, TC> b;
-    std::memcpy(&b, &L.a, sizeof(b));
-    seg_patch<T, TC>(b, L, w);
-    if (a.resmax || a.glo || a.Ft || a.dev || !seg_same_args(a, b))
-        return fail(BIOT_ERR_CUDA, "segment program: a sweep is not reproduced by its job word");
-    *out = w;
-    return BIOT_OK;
-}
-
-// The program of recorded sweeps rec[i0 .. i1) (one storage family).
-int seg_build(const biot_ctx *h, const std::vector<SweepJob> &rec, size_t i0, size_t i1, SegProg &prog)
-{
-    prog.fam = rec[i0].tkind == 0 ? 0 : 1;
-    prog.cs = 1;
-    prog.lev.clear();
-    prog.job.clear();
-    std::vector<int> lvl;  // level of each record
-    for (size_t k = i0; k < i1; k++) {
-        const SweepJob &j = rec[k];
-        const int l = j.level;
-        int rel = (int)(std::find(lvl.begin(), lvl.end(), l) - lvl.begin());
-        if (rel == (int)lvl.size()) {
-            if (rel > SEGJ_LEVEL) return fail(BIOT_ERR_CUDA, "segment program: too many levels");
-            SegLevel L;
-            std::memset(&L, 0, sizeof(L));
-            L.tkind = j.tkind;
-            if (j.tkind == 0) L.a.dd = j.dd;
-            else if (j.tkind == 1) L.a.fd = j.fd;
-            else L.a.ff = j.ff;
-            L.buf[0] = h->lv[l].g[0];
-            L.buf[1] = h->lv[l].g[1];
-            if (l > 0) {
-                L.cbuf[0] = h->lv[l - 1].g[0];
-                L.cbuf[1] = h->lv[l - 1].g[1];
-                L.crc = h->lv[l - 1].r;
-            }
-            prog.lev.push_back(L);
-            lvl.push_back(l);
-        }
-        const SegLevel &L = prog.lev[rel];
-        if (L.tkind != j.tkind) return fail(BIOT_ERR_CUDA, "segment program: a level changed its storage kind");
-        unsigned w = 0;
-        int rc = j.tkind == 0 ? seg_word<double, double>(h, j.dd, l, L, rel, &w)
-               : j.tkind == 1 ? seg_word<float, double>(h, j.fd, l, L, rel, &w)
-                              : seg_word<float, float>(h, j.ff, l, L, rel, &w);
-        if (rc) return rc;
-        prog.job.push_back(w);
-        prog.cs = std::max(prog.cs, std::min(SEG_CLUSTER, seg_tiles_of(h, l)));
+    for (int l = 0; l <= s; l++) h->lv[l].hist_valid = 1;  // as after the level's own sweeps
+    if (h->rec) {
+        if (!h->resrec) return fail(BIOT_ERR_CUDA, "resident cycle recorded without a program list");
+        SweepJob m{};
+        m.tkind = 2;
+        m.variant = SWEEP_V_RESIDENT | (h->P.ne_fixed > 0 ? SWEEP_V_NOGHOST : 0);
+        m.level = s;
+        m.res = (int)h->resrec->size();
+        h->resrec->push_back(R);
+        h->rec->push_back(m);
+        return BIOT_OK;
     }
-    if (prog.lev.size() > (size_t)SEG_MAX_LEVELS || prog.job.size() > (size_t)SEG_MAX_JOBS)
-        return fail(BIOT_ERR_CUDA, "segment program: too many levels or sweeps for one launch");
-    return BIOT_OK;
-}
-
-// Append program g to the launch parameters P (false: P is full).
-bool seg_pack(SegParams &P, const SegProg &g)
-{
-    if (P.nprog >= SEG_MAX_PROGS || P.lev0[P.nprog] + (int)g.lev.size() > SEG_MAX_LEVELS ||
-        P.job0[P.nprog] + (int)g.job.size() > SEG_MAX_JOBS)
-        return false;
-    const int p = P.nprog;
-    std::copy(g.lev.begin(), g.lev.end(), P.lev + P.lev0[p]);
-    std::copy(g.job.begin(), g.job.end(), P.job + P.job0[p]);
-    P.lev0[p + 1] = P.lev0[p] + (int)g.lev.size();
-    P.job0[p + 1] = P.job0[p] + (int)g.job.size();
-    P.nprog = p + 1;
-    return true;
-}
-
-cudaError_t seg_launch(int fam, const SegParams &P, int cs, cudaStream_t s)
-{
-    return fam == 0 ? launch_sweep_segment<double>(P, cs, s) : launch_sweep_segment<float>(P, cs, s);
-}
-
-int vcycle(biot_ctx *h, int l, bool zero_start, bool prolong_first, int kind);
-
-// The V-cycle from level l down (a coarse-grid correction, zero start) as
-// segments.  Single instance: one launch per run of one storage family, except
-// that a run of the coarsest level's smoothing sweeps alone, FP64 and at most
-// SWEEP_CHAIN_MAX^2 cells, keeps the chained launch.  Batch (record mode): one
-// recorded job per run, whose program goes to segrec.
-int seg_vcycle(biot_ctx *h, int l)
-{
-    std::vector<SweepJob> rec;
-    std::vector<SweepJob> *outer = h->rec;
-    h->rec = &rec;
-    h->in_seg = true;
-    int rc = vcycle(h, l, true, false, BIOT_CYCLE_V);
-    h->rec = outer;
-    h->in_seg = false;
-    if (rc) return rc;
-    std::unique_ptr<SegParams> P;
-    for (size_t i = 0; i < rec.size();) {
-        const int fam = rec[i].tkind == 0 ? 0 : 1;
-        size_t j = i;
-        while (j < rec.size() && (rec[j].tkind == 0 ? 0 : 1) == fam) j++;
-        SegProg prog;
-        if ((rc = seg_build(h, rec, i, j, prog))) return rc;
-        if (outer) {
-            if (!h->segrec) return fail(BIOT_ERR_CUDA, "segment recorded without a program list");
-            SweepJob m{};
-            m.tkind = fam == 0 ? 0 : 2;
-            m.variant = SWEEP_V_SEGMENT | (h->P.ne_fixed > 0 ? SWEEP_V_NOGHOST : 0);
-            m.level = rec[i].level;
-            m.seg = (int)h->segrec->size();
-            h->segrec->push_back(std::move(prog));
-            outer->push_back(m);
-        } else {
-            bool chain = fam == 0 && h->lv[0].nx <= SWEEP_CHAIN_MAX && h->lv[0].ny <= SWEEP_CHAIN_MAX && j - i > 1;
-            for (size_t k = i; k < j && chain; k++) chain = rec[k].level == 0 && rec[k].dd.mode == SWEEP_SMOOTH;
-            if (chain) {
-                CUDA_TRY((launch_sweep_chain<double, double>(rec[i].dd, (int)(j - i), h->stream)));
-            } else {
-                if (!P) P.reset(new (std::nothrow) SegParams());
-                if (!P) return fail(BIOT_ERR_OOM, "segment launch parameters");
-                P->nprog = 0;
-                P->ghosts = h->P.ne_fixed > 0 ? 0 : 1;
-                P->lev0[0] = P->job0[0] = 0;
-                if (!seg_pack(*P, prog)) return fail(BIOT_ERR_CUDA, "segment program too large for one launch");
-                CUDA_TRY(seg_launch(fam, *P, prog.cs, h->stream));
-            }
-            h->launches++;
-        }
-        i = j;
-    }
+    std::unique_ptr<ResParams> PP(new (std::nothrow) ResParams());
+    if (!PP) return fail(BIOT_ERR_OOM, "resident launch parameters");
+    PP->nprog = 1;
+    PP->cs = R.cs;
+    PP->ghosts = h->P.ne_fixed > 0 ? 0 : 1;
+    PP->p[0] = P;
+    CUDA_TRY(launch_resident(*PP, R.smem, h->stream));
+    h->launches++;
     return BIOT_OK;
 }
 
@@ -753,19 +727,11 @@ int seg_vcycle(biot_ctx *h, int l)
 // followed by a V-cycle (F).
 int vcycle(biot_ctx *h, int l, bool zero_start, bool prolong_first = false, int kind = BIOT_CYCLE_V)
 {
-    // a coarse-grid correction from the segment's start level down: as segments
-    // (a single instance keeps the chained coarsest level when that is all)
-    if (kind == BIOT_CYCLE_V && zero_start && !prolong_first && !h->in_seg && l == seg_start(h, h->cold_solve) &&
-        (h->rec || l > 0))
-        return seg_vcycle(h, l);
+    // a small level's correction problem in one launch
+    if (l < h->L - 1 && !prolong_first && l <= res_start(h, h->cold_solve, kind)) return res_cycle(h, l, zero_start, kind);
     const int K = sweeps_of(&h->P, l);
     const bool fine = (l == h->L - 1);
     int rc;
-    // the coarsest level's 2K sweeps, when it is a small FP64 level below the
-    // finest, in one launch (a batch records them one by one)
-    const Level &Lv = h->lv[l];
-    if (l == 0 && !fine && !h->rec && Lv.fp64 && Lv.nx <= SWEEP_CHAIN_MAX && Lv.ny <= SWEEP_CHAIN_MAX && !prolong_first)
-        return sweep(h, 0, SWEEP_SMOOTH, zero_start, false, false, 2 * K);
     for (int k = 0; k < K; k++)
         if ((rc = sweep(h, l, SWEEP_SMOOTH, zero_start && k == 0, prolong_first && k == 0, false))) return rc;
     if (l > 0) {
@@ -1929,16 +1895,12 @@ constexpr long BATCH_TILE_MAX_CELLS = 128L * 128L;
 // Whether the depth groups' branches of the step graph run at descending stream
 // priorities, deepest first.
 constexpr bool BATCH_BRANCH_PRIORITIES = true;
-// Whether a batch runs the 2K sweeps of each instance's FP64 coarsest level as
-// one segment launch (one cluster per instance) rather than 2K phase launches.
-constexpr bool BATCH_COARSEST_SEGMENT = true;
 long batch_tile_max_cells() { return BATCH_TILE_MAX_CELLS; }
 
-// One sweep of the static schedule of an instance, or one segment (fam >= 0:
-// a run of sweeps of one storage family, launched as one program).
+// One sweep of the static schedule of an instance, or one resident V-cycle.
 struct PlanOp {
     int level, mode, key;
-    int fam = -1;
+    bool resident = false;
 };
 
 // Mirror of vcycle(): the sweeps of one V-cycle from level l down, with their
@@ -1963,13 +1925,12 @@ void plan_vcycle(const biot_ctx *h, int l, int K, int Dmax, std::vector<PlanOp> 
         out.push_back({l, SWEEP_SMOOTH, l == 0 ? bottom + K + k : bottom + 2 * K + (l - 1) * K + k});
 }
 
-// The ops of the segments of one V-cycle's plan collapsed as seg_vcycle
-// records them: the ops of the levels at or below the segment's start level are
-// contiguous (the coarse-grid correction), and each run of one storage family
-// among them becomes one op at the key of its first sweep.
-void plan_segments(const biot_ctx *h, std::vector<PlanOp> &ops)
+// The ops of the resident V-cycle of one V-cycle's plan collapsed as res_cycle
+// records it: the ops of the levels at or below its start level are contiguous
+// (the coarse-grid correction) and become one op at the key of the first.
+void plan_resident(const biot_ctx *h, std::vector<PlanOp> &ops)
 {
-    const int s = seg_start(h, false);
+    const int s = res_start(h, false);
     if (s < 0) return;
     std::vector<PlanOp> out;
     for (size_t i = 0; i < ops.size();) {
@@ -1977,13 +1938,10 @@ void plan_segments(const biot_ctx *h, std::vector<PlanOp> &ops)
             out.push_back(ops[i++]);
             continue;
         }
-        const int fam = h->lv[ops[i].level].fp64 ? 0 : 1;
         PlanOp m = ops[i];
-        m.fam = fam;
-        size_t j = i;
-        while (j < ops.size() && ops[j].level <= s && (h->lv[ops[j].level].fp64 ? 0 : 1) == fam) j++;
+        m.resident = true;
         out.push_back(m);
-        i = j;
+        while (i < ops.size() && ops[i].level <= s) i++;
     }
     ops.swap(out);
 }
@@ -2011,12 +1969,12 @@ int level_variant(const biot_ctx *h, int l, int mode)
 
 int op_tkind(const biot_ctx *h, const PlanOp &o)
 {
-    return o.fam >= 0 ? (o.fam == 0 ? 0 : 2) : level_tkind(h, o.level);
+    return o.resident ? 2 : level_tkind(h, o.level);
 }
 
 int op_variant(const biot_ctx *h, const PlanOp &o)
 {
-    if (o.fam >= 0) return SWEEP_V_SEGMENT | (h->P.ne_fixed > 0 ? SWEEP_V_NOGHOST : 0);
+    if (o.resident) return SWEEP_V_RESIDENT | (h->P.ne_fixed > 0 ? SWEEP_V_NOGHOST : 0);
     return level_variant(h, o.level, o.mode);
 }
 
@@ -2144,9 +2102,9 @@ int batch_plan(biot_batch_s *b)
         const int up = Dg * (b->K + 1) + 2 * b->K + Dg * b->K;
         std::vector<PlanOp> cyc;
         plan_vcycle(b->inst[i], b->inst[i]->L - 1, b->K, Dg, cyc);
-        plan_segments(b->inst[i], cyc);
+        plan_resident(b->inst[i], cyc);
         for (int c = 0; c < b->ne; c++)
-            for (const PlanOp &o : cyc) ops[i].push_back({o.level, o.mode, c * up + o.key, o.fam});
+            for (const PlanOp &o : cyc) ops[i].push_back({o.level, o.mode, c * up + o.key, o.resident});
         b->nops[i] = ops[i].size();
         int &mk = maxkey[b->group_of[i]];
         for (const PlanOp &o : ops[i]) mk = o.key > mk ? o.key : mk;
@@ -2171,7 +2129,7 @@ int batch_plan(biot_batch_s *b)
                     grp.push_back(s);
                 }
                 if (grp.empty()) continue;
-                if (v & SWEEP_V_SEGMENT) {  // segments: one program per job, no work items
+                if (v & SWEEP_V_RESIDENT) {  // resident V-cycles: one program per job, no work items
                     BatchLaunch L{tk, v, b->slots[tk].size(), b->items.size(), (int)grp.size(), 0, g};
                     for (const BatchSlot &sl : grp) b->slots[tk].push_back(sl);
                     b->launches.push_back(L);
@@ -2289,40 +2247,29 @@ cudaError_t batch_launch_typed(biot_batch_s *b, const BatchLaunch &L, std::vecto
     return it == it_end ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// A planned launch of segments: the programs of its jobs packed into as few
-// launches as the parameter block allows (*nl: how many).
-cudaError_t batch_launch_segments(biot_batch_s *b, const BatchLaunch &L, std::vector<std::vector<SweepJob>> &rec,
-                                  std::vector<std::vector<SegProg>> &segrec, cudaStream_t stream, long *nl)
+// A planned launch of resident V-cycles, one cluster per instance: at most
+// RES_MAX_PROGS programs per launch (*nl: how many launches).
+cudaError_t batch_launch_resident(biot_batch_s *b, const BatchLaunch &L, std::vector<std::vector<SweepJob>> &rec,
+                                  std::vector<std::vector<ResLaunch>> &resrec, cudaStream_t stream, long *nl)
 {
-    std::unique_ptr<SegParams> P(new (std::nothrow) SegParams());
+    std::unique_ptr<ResParams> P(new (std::nothrow) ResParams());
     if (!P) return cudaErrorMemoryAllocation;
-    const int fam = L.tkind == 0 ? 0 : 1;
-    int cs = 1;
-    auto reset = [&]() {
-        P->nprog = 0;
+    for (int k0 = 0; k0 < L.njobs; k0 += RES_MAX_PROGS) {
+        const int n = std::min(RES_MAX_PROGS, L.njobs - k0);
+        size_t smem = 0;
+        P->nprog = n;
+        P->cs = 1;
         P->ghosts = (L.variant & SWEEP_V_NOGHOST) ? 0 : 1;
-        P->lev0[0] = P->job0[0] = 0;
-        cs = 1;
-    };
-    reset();
-    for (int k = 0; k < L.njobs; k++) {
-        const BatchSlot &sl = b->slots[L.tkind][L.job_off + k];
-        const int gi = rec[sl.inst][sl.op].seg;
-        if (gi < 0 || gi >= (int)segrec[sl.inst].size()) return cudaErrorInvalidValue;
-        const SegProg &g = segrec[sl.inst][gi];
-        if (g.fam != fam) return cudaErrorInvalidValue;
-        if (!seg_pack(*P, g)) {
-            if (P->nprog == 0) return cudaErrorInvalidValue;
-            cudaError_t e = seg_launch(fam, *P, cs, stream);
-            if (e != cudaSuccess) return e;
-            (*nl)++;
-            reset();
-            if (!seg_pack(*P, g)) return cudaErrorInvalidValue;
+        for (int k = 0; k < n; k++) {
+            const BatchSlot &sl = b->slots[L.tkind][L.job_off + k0 + k];
+            const int ri = rec[sl.inst][sl.op].res;
+            if (ri < 0 || ri >= (int)resrec[sl.inst].size()) return cudaErrorInvalidValue;
+            const ResLaunch &R = resrec[sl.inst][ri];
+            P->p[k] = R.prog;
+            P->cs = std::max(P->cs, R.cs);
+            smem = std::max(smem, R.smem);
         }
-        cs = std::max(cs, g.cs);
-    }
-    if (P->nprog > 0) {
-        cudaError_t e = seg_launch(fam, *P, cs, stream);
+        cudaError_t e = launch_resident(*P, smem, stream);
         if (e != cudaSuccess) return e;
         (*nl)++;
     }
@@ -2334,7 +2281,7 @@ int batch_capture(biot_batch_s *b, int par)
 {
     const int n = (int)b->inst.size();
     std::vector<std::vector<SweepJob>> rec(n);
-    std::vector<std::vector<SegProg>> segrec(n);
+    std::vector<std::vector<ResLaunch>> resrec(n);
     std::vector<FlowRec> frec;
     std::vector<long> l0(n), c0(n);
     CUDA_TRY(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
@@ -2346,11 +2293,11 @@ int batch_capture(biot_batch_s *b, int par)
         c0[i] = h->total_cycles;
         h->rec = &rec[i];
         h->frec = &frec;
-        h->segrec = &segrec[i];
+        h->resrec = &resrec[i];
         rc = advance(h);  // flow steps and sweeps are recorded, launched below for all instances
         h->rec = nullptr;
         h->frec = nullptr;
-        h->segrec = nullptr;
+        h->resrec = nullptr;
         if (!rc && frec.size() != (size_t)i + 1) rc = fail(BIOT_ERR_CUDA, "batched schedule: flow step not recorded");
         nl += h->launches - l0[i];
         if (!rc && rec[i].size() != b->nops[i]) rc = fail(BIOT_ERR_CUDA, "batched schedule does not match the recorded sweeps");
@@ -2395,9 +2342,9 @@ int batch_capture(biot_batch_s *b, int par)
     for (size_t k = 0; k < b->launches.size() && !rc; k++) {
         const BatchLaunch &L = b->launches[k];
         const cudaStream_t st = fork ? b->branch[L.group] : b->stream;
-        if (L.variant & SWEEP_V_SEGMENT) {
-            cudaError_t e = batch_launch_segments(b, L, rec, segrec, st, &nl);
-            if (e != cudaSuccess) rc = fail(BIOT_ERR_CUDA, std::string("batched segment launch: ") + cudaGetErrorString(e));
+        if (L.variant & SWEEP_V_RESIDENT) {
+            cudaError_t e = batch_launch_resident(b, L, rec, resrec, st, &nl);
+            if (e != cudaSuccess) rc = fail(BIOT_ERR_CUDA, std::string("batched resident launch: ") + cudaGetErrorString(e));
             continue;
         }
         cudaError_t e = L.tkind == 0 ? batch_launch_typed<double, double>(b, L, rec, st)
@@ -2509,12 +2456,12 @@ int biot_batch_create(int count, const biot_params *params, const biot_side *sid
             return fail(rc, msg);
         }
         b->inst.push_back(h);
-        h->batched = BATCH_COARSEST_SEGMENT;
         if (cudaStreamSynchronize(h->stream) != cudaSuccess) {
             batch_release(b);
             return fail(BIOT_ERR_CUDA, "instance set-up failed");
         }
         h->stream = b->stream;
+        h->batched = true;
         b->Dmax = h->L - 1 > b->Dmax ? h->L - 1 : b->Dmax;
     }
     int rc = batch_plan(b);

@@ -2,5 +2,5 @@
 // whose next coarser level is also FP32, and the per-cell field kernels).
 #include "instantiate.h"
 
-BIOT_SWEEP_MOM(float, float)
+BIOT_SWEEP_SINGLE(float, float)
 BIOT_FIELDS(float)

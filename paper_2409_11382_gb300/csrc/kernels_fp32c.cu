@@ -3,4 +3,4 @@
 // its own so that the build compiles it in parallel with the others.
 #include "instantiate.h"
 
-BIOT_SWEEP_MOM(float, double)
+BIOT_SWEEP_SINGLE(float, double)

@@ -3,8 +3,8 @@
 // changes the rounding.
 #include "instantiate.h"
 
-BIOT_SWEEP_MOM(double, double)
-BIOT_SEGMENT(double)
+BIOT_SWEEP_SINGLE(double, double)
+BIOT_SWEEP_BATCH(double, double)
 BIOT_FIELDS(double)
 
 // Stopping test of one V-cycle (tolerance mode, inside a CUDA graph):
