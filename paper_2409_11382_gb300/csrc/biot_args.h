@@ -278,6 +278,20 @@ inline int sweep_strip_rows(int nx, int ny, int slots)
         if (ty <= cap || waves >= 64) return (int)ty;
     }
 }
+// Rows per strip of the packed sweep (sweep_pair.cuh): nsx strips side by side over
+// `rows` rows, `slots` resident warps.  Whole waves of strips, as few as give strips
+// of at most 64 rows: a strip's four extra rows cost least when it is tall, and one
+// wave of 158-row strips ends with SMs idle (4096^2: 8.13 ms per step in one wave,
+// 7.70 in three; 32, 48, 64 and 96 rows at most: 7.72, 7.71, 7.73, 7.87).  Even.
+inline int pair_rows(int nsx, int rows, int slots)
+{
+    for (int waves = 1;; waves++) {
+        const int blocks = waves * slots / nsx > 0 ? waves * slots / nsx : 1;
+        int ty = (rows + blocks - 1) / blocks;
+        ty += ty & 1;
+        if (ty <= 64 || waves >= 64) return ty < 4 ? 4 : ty;
+    }
+}
 template <typename T> cudaError_t launch_sexp(const SexpArgs<T> &a, cudaStream_t s);
 template <typename T> cudaError_t launch_force(const ForceArgs<T> &a, cudaStream_t s);
 template <typename T> cudaError_t launch_readout(const ReadoutArgs<T> &a, cudaStream_t s);

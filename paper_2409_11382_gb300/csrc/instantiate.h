@@ -4,6 +4,7 @@
 #include "field_kernels.cuh"
 #include "sweep_batch.cuh"
 #include "sweep_mom.cuh"
+#include "sweep_pair.cuh"
 
 // The single-instance and the batched sweeps of a storage pair: units of their own
 // for FP32, so that the build compiles them in parallel.
