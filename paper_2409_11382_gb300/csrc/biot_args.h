@@ -76,7 +76,10 @@ struct SweepItem {
 
 // Storage kind of a sweep launch (bit flags).
 enum { SWEEP_V_COARSE = 1, SWEEP_V_LO = 2, SWEEP_V_RESTRICT = 4, SWEEP_V_NOGHOST = 8, SWEEP_V_TILE = 16,
-       SWEEP_V_DEV16 = 32, SWEEP_V_DEVBF16 = 64, SWEEP_V_RESIDENT = 128 };
+       SWEEP_V_DEV16 = 32, SWEEP_V_DEVBF16 = 64, SWEEP_V_RESIDENT = 128,
+       // packed strips (sweep_pair.cuh), with the prolongated correction added or from zero
+       SWEEP_V_PAIR = 256, SWEEP_V_PROL = 512, SWEEP_V_ZERO = 1024,
+       SWEEP_V_SHAPE = SWEEP_V_TILE | SWEEP_V_PAIR | SWEEP_V_PROL | SWEEP_V_ZERO };  // chosen by the plan, not by the sweep
 // Tile sweeps: levels of at most SWEEP_TILE_CELLS cells (single instance); tile
 // shape per storage type.  The fused flow step works on FLOW_TILE_X x FLOW_TILE_Y tiles.
 constexpr long SWEEP_TILE_CELLS = 256L * 256L;
@@ -283,15 +286,35 @@ inline int sweep_strip_rows(int nx, int ny, int slots)
 // of at most 64 rows: a strip's four extra rows cost least when it is tall, and one
 // wave of 158-row strips ends with SMs idle (4096^2: 8.13 ms per step in one wave,
 // 7.70 in three; 32, 48, 64 and 96 rows at most: 7.72, 7.71, 7.73, 7.87).  Even.
+constexpr int PAIR_WARPS = 4;              // warps of a CTA, one strip each
+constexpr int PAIR_COLS = 60;              // columns a strip writes: 64 less two on each side
+constexpr int PAIR_FX = 16, PAIR_FY = 2;   // frame tiles along the top and bottom; the sides take them transposed
+constexpr int PAIR_CTAS = 3;               // resident CTAs per SM (its register bound)
+inline int pair_rows_for(int nsx, int rows, int warps)
+{
+    const int blocks = warps / nsx > 0 ? warps / nsx : 1;
+    int ty = (rows + blocks - 1) / blocks;
+    ty += ty & 1;
+    return ty < 4 ? 4 : ty;
+}
 inline int pair_rows(int nsx, int rows, int slots)
 {
     for (int waves = 1;; waves++) {
-        const int blocks = waves * slots / nsx > 0 ? waves * slots / nsx : 1;
-        int ty = (rows + blocks - 1) / blocks;
-        ty += ty & 1;
-        if (ty <= 64 || waves >= 64) return ty < 4 ? 4 : ty;
+        const int ty = pair_rows_for(nsx, rows, waves * slots);
+        if (ty <= 64 || waves >= 64) return ty;
     }
 }
+// CTAs of the strips of an nx x ny level in row blocks of TY rows, and of its frame.
+__host__ __device__ inline int pair_strips_x(int nx) { return (nx - 4 + PAIR_COLS - 1) / PAIR_COLS; }
+__host__ __device__ inline int pair_strip_ctas(int nx, int ny, int TY)
+{
+    return (pair_strips_x(nx) * ((ny - 4 + TY - 1) / TY) + PAIR_WARPS - 1) / PAIR_WARPS;
+}
+__host__ __device__ inline int pair_frame_ctas(int nx, int ny)
+{
+    return 2 * ((nx + PAIR_FX - 1) / PAIR_FX) + 2 * ((ny + PAIR_FX - 1) / PAIR_FX);
+}
+
 template <typename T> cudaError_t launch_sexp(const SexpArgs<T> &a, cudaStream_t s);
 template <typename T> cudaError_t launch_force(const ForceArgs<T> &a, cudaStream_t s);
 template <typename T> cudaError_t launch_readout(const ReadoutArgs<T> &a, cudaStream_t s);

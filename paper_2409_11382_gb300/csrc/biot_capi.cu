@@ -559,8 +559,8 @@ int res_min_cells(const biot_ctx *h, bool fp64) { return !fp64 ? 256 : h->batche
 // 0.528 and 0.554 ms at 256^2, 1.62 and 1.66 ms at 1024^2) and 2048 cells in FP64
 // (against 1024: 0.600 and 0.686 ms per 64^2 FP64 step); with an FP32 coarsest
 // level 32^2, where 64^2 gains 1 % (0.793 and 0.801 ms at 512^2).  A batch's phase
-// launches fill the GPU, and a cluster holds SMs that they would use: 16^2 (6.63
-// ms per step of the 64-instance workload, 32^2: 6.77, 64^2: 7.75).
+// launches fill the GPU, and a cluster holds SMs that they would use: 16^2 (with
+// the general strips 6.63 ms per step of the 64-instance workload, 32^2: 6.77, 64^2: 7.75).
 long res_max_cells(const biot_ctx *h, bool fp64)
 {
     if (h->batched) return 256;
@@ -1901,6 +1901,8 @@ long batch_tile_max_cells() { return BATCH_TILE_MAX_CELLS; }
 struct PlanOp {
     int level, mode, key;
     bool resident = false;
+    int fetch = 0;          // SWEEP_V_PROL / SWEEP_V_ZERO as the sweep's loads form its iterate
+    bool measured = false;  // the sweep that measures the residual
 };
 
 // Mirror of vcycle(): the sweeps of one V-cycle from level l down, with their
@@ -1916,13 +1918,16 @@ void plan_vcycle(const biot_ctx *h, int l, int K, int Dmax, std::vector<PlanOp> 
     // level runs its own count Kl <= K of the sweeps of each leg
     const int Kl = sweeps_of(&h->P, l);
     const int bottom = Dmax * (K + 1);  // first key of the coarsest sweeps
-    for (int k = 0; k < Kl; k++) out.push_back({l, SWEEP_SMOOTH, l == 0 ? bottom + k : (Dmax - l) * (K + 1) + k});
+    const bool fine = l == h->L - 1;
+    for (int k = 0; k < Kl; k++)
+        out.push_back({l, SWEEP_SMOOTH, l == 0 ? bottom + k : (Dmax - l) * (K + 1) + k, false, k == 0 && !fine ? (int)SWEEP_V_ZERO : 0});
     if (l > 0) {
         out.push_back({l, SWEEP_RESTRICT, (Dmax - l) * (K + 1) + K});
         plan_vcycle(h, l - 1, K, Dmax, out);
     }
     for (int k = 0; k < Kl; k++)
-        out.push_back({l, SWEEP_SMOOTH, l == 0 ? bottom + K + k : bottom + 2 * K + (l - 1) * K + k});
+        out.push_back({l, SWEEP_SMOOTH, l == 0 ? bottom + K + k : bottom + 2 * K + (l - 1) * K + k, false,
+                       k == 0 && l > 0 ? (int)SWEEP_V_PROL : 0, fine && k == Kl - 1});
 }
 
 // The ops of the resident V-cycle of one V-cycle's plan collapsed as res_cycle
@@ -1975,7 +1980,15 @@ int op_tkind(const biot_ctx *h, const PlanOp &o)
 int op_variant(const biot_ctx *h, const PlanOp &o)
 {
     if (o.resident) return SWEEP_V_RESIDENT | (h->P.ne_fixed > 0 ? SWEEP_V_NOGHOST : 0);
-    return level_variant(h, o.level, o.mode);
+    const int v = level_variant(h, o.level, o.mode);
+    // packed strips where they take the sweep (pair_takes): FP32 above FP32, double-float
+    // first moments on the finest level only, no deviation store, no measured residual
+    const Level &Lv = h->lv[o.level];
+    const bool fine = o.level == h->L - 1;
+    const bool pair = !(v & (SWEEP_V_TILE | SWEEP_V_DEV16 | SWEEP_V_DEVBF16)) && (v & SWEEP_V_NOGHOST) && !o.measured &&
+                      level_tkind(h, o.level) == 2 && ((v & SWEEP_V_LO) != 0) == fine && Lv.nx % 4 == 0 && Lv.ny % 2 == 0 &&
+                      Lv.nx >= 64 && Lv.ny >= 8;
+    return pair ? v | SWEEP_V_PAIR | o.fetch : v;
 }
 
 // Strip heights of one batched launch (levels of nx x ny cells): the fewest whole
@@ -2002,6 +2015,27 @@ std::vector<int> batch_strip_rows(const std::vector<std::pair<int, int>> &dims, 
             if (t < 2) t = 2;
             ty[g] = (int)t;
             if (t > cap) ok = false;
+        }
+        if (ok) break;
+    }
+    return ty;
+}
+
+// Rows per strip of a batched launch of packed strips: the fewest whole waves of
+// `slots` warps whose share per level gives strips of at most 64 rows.  (With packed
+// strips a step of the 64-instance workload takes 4.83 ms, with the general strips
+// 6.63 ms.)
+std::vector<int> batch_pair_rows(const std::vector<std::pair<int, int>> &dims, int slots)
+{
+    double cells = 0;
+    for (const auto &d : dims) cells += (double)d.first * d.second;
+    std::vector<int> ty(dims.size(), 4);
+    for (int waves = 1; waves <= 64; waves++) {
+        bool ok = true;
+        for (size_t g = 0; g < dims.size(); g++) {
+            const double share = (double)waves * slots * ((double)dims[g].first * dims[g].second) / cells;
+            ty[g] = pair_rows_for(pair_strips_x(dims[g].first), dims[g].second - 4, (int)share);
+            ok = ok && ty[g] <= 64;
         }
         if (ok) break;
     }
@@ -2039,7 +2073,7 @@ struct BatchSlot {
 struct biot_batch_s {
     std::vector<biot_ctx *> inst;
     cudaStream_t stream = nullptr;
-    int K = 0, ne = 0, Dmax = 0;
+    int K = 0, ne = 0, Dmax = 0, sms = 1;
     std::vector<BatchLaunch> launches;            // in issue order
     std::vector<BatchSlot> slots[3];              // per tkind: the recorded sweep of each job
     std::vector<SweepItem> items;
@@ -2104,11 +2138,14 @@ int batch_plan(biot_batch_s *b)
         plan_vcycle(b->inst[i], b->inst[i]->L - 1, b->K, Dg, cyc);
         plan_resident(b->inst[i], cyc);
         for (int c = 0; c < b->ne; c++)
-            for (const PlanOp &o : cyc) ops[i].push_back({o.level, o.mode, c * up + o.key, o.resident});
+            for (const PlanOp &o : cyc) ops[i].push_back({o.level, o.mode, c * up + o.key, o.resident, o.fetch, o.measured && c == b->ne - 1});
         b->nops[i] = ops[i].size();
         int &mk = maxkey[b->group_of[i]];
         for (const PlanOp &o : ops[i]) mk = o.key > mk ? o.key : mk;
     }
+    int dev = 0;
+    CUDA_TRY(cudaGetDevice(&dev));
+    CUDA_TRY(cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev));
     b->launches.clear();
     b->items.clear();
     for (int t = 0; t < 3; t++) b->slots[t].clear();
@@ -2119,8 +2156,16 @@ int batch_plan(biot_batch_s *b)
         if (b->group_of[i] == g)
             for (size_t j = 0; j < ops[i].size(); j++) bykey[ops[i][j].key].push_back({i, (int)j});
     for (int key = 0; key <= maxkey[g]; key++) {
-        for (int tk = 0; tk < 3; tk++) {
-            for (int v = 0; v < 256; v++) {  // every combination of the SWEEP_V_* flags
+        std::vector<std::pair<int, int>> kinds;  // the (storage kind, variant) pairs of this phase
+        for (const BatchSlot &s : bykey[key]) {
+            const PlanOp &o = ops[s.inst][s.op];
+            const std::pair<int, int> k{op_tkind(b->inst[s.inst], o), op_variant(b->inst[s.inst], o)};
+            if (std::find(kinds.begin(), kinds.end(), k) == kinds.end()) kinds.push_back(k);
+        }
+        std::sort(kinds.begin(), kinds.end());
+        for (const auto &kind : kinds) {
+            {
+                const int tk = kind.first, v = kind.second;
                 std::vector<BatchSlot> grp;
                 for (const BatchSlot &s : bykey[key]) {
                     const biot_ctx *h = b->inst[s.inst];
@@ -2135,12 +2180,19 @@ int batch_plan(biot_batch_s *b)
                     b->launches.push_back(L);
                     continue;
                 }
-                const bool tile = (v & SWEEP_V_TILE) != 0;
-                const int slots = tile ? 1 : tkind_slots(tk, v & ~SWEEP_V_TILE);
+                const bool tile = (v & SWEEP_V_TILE) != 0, pair = (v & SWEEP_V_PAIR) != 0;
+                const int slots = tile || pair ? 1 : tkind_slots(tk, v);
                 if (!slots) return fail(BIOT_ERR_CUDA, "occupancy query of the batched sweep kernel failed");
                 BatchLaunch L{tk, v, b->slots[tk].size(), b->items.size(), (int)grp.size(), 0, g};
                 std::vector<int> tys;
-                if (!tile) {
+                if (pair) {
+                    std::vector<std::pair<int, int>> dims;
+                    for (const BatchSlot &s : grp) {
+                        const Level &Lv = b->inst[s.inst]->lv[ops[s.inst][s.op].level];
+                        dims.push_back({Lv.nx, Lv.ny});
+                    }
+                    tys = batch_pair_rows(dims, b->sms * PAIR_CTAS * PAIR_WARPS);
+                } else if (!tile) {
                     std::vector<std::pair<int, int>> dims;
                     for (const BatchSlot &s : grp) {
                         const Level &Lv = b->inst[s.inst]->lv[ops[s.inst][s.op].level];
@@ -2156,6 +2208,9 @@ int batch_plan(biot_batch_s *b)
                         sweep_tile_shape(tk == 0, &tx, &ty);
                         for (int by = 0; by < (Lv.ny + ty - 1) / ty; by++)
                             for (int bx = 0; bx < (Lv.nx + tx - 1) / tx; bx++) b->items.push_back({(int)g, bx, by, 0});
+                    } else if (pair) {  // the CTAs of the level's packed sweep: strips, then its frame
+                        const int n = pair_strip_ctas(Lv.nx, Lv.ny, tys[g]) + pair_frame_ctas(Lv.nx, Lv.ny);
+                        for (int i = 0; i < n; i++) b->items.push_back({(int)g, 0, 0, tys[g]});
                     } else {  // strips sized so that the launch fills whole waves of the GPU
                         const int ty = tys[g];
                         const int sx = (Lv.nx + BATCH_STRIP_COLS - 1) / BATCH_STRIP_COLS, sy = (Lv.ny + ty - 1) / ty;
@@ -2315,7 +2370,7 @@ int batch_capture(biot_batch_s *b, int par)
         for (int j = 0; j < L.njobs && !rc; j++) {
             const BatchSlot &sl = b->slots[L.tkind][L.job_off + j];
             const SweepJob &r = rec[sl.inst][sl.op];
-            if (r.tkind != L.tkind || r.variant != (L.variant & ~SWEEP_V_TILE))
+            if (r.tkind != L.tkind || r.variant != (L.variant & ~SWEEP_V_SHAPE))
                 rc = fail(BIOT_ERR_CUDA, "batched schedule: a recorded sweep differs from its planned kind");
         }
     }

@@ -117,9 +117,16 @@ struct SlotsRun {
     static int run() { return BatchKernel<T, TC, KIND, LO, RS>::slots(); }
 };
 
+// The packed strips of a batched launch (sweep_pair.cuh).
+cudaError_t launch_pair_batch(int v, const BatchParams<float, float> &P, cudaStream_t s);
+
 template <typename T, typename TC>
 cudaError_t launch_sweep_batch_impl(int v, const BatchParams<T, TC> &P, cudaStream_t s)
 {
+    if (v & SWEEP_V_PAIR) {
+        if constexpr (sizeof(T) == 4 && sizeof(TC) == 4) return launch_pair_batch(v, P, s);
+        else return cudaErrorInvalidValue;
+    }
     return dispatch_kind<T, TC, BatchRun>(v & SWEEP_V_COARSE, v & SWEEP_V_LO, v & SWEEP_V_RESTRICT,
                                          !(v & SWEEP_V_NOGHOST), (v & SWEEP_V_DEV16) ? 1 : (v & SWEEP_V_DEVBF16) ? 2 : 0,
                                          (v & SWEEP_V_TILE) != 0, P, s);

@@ -25,6 +25,7 @@
 // ms).  Per time step: 4096^2 11.4 -> 7.7 ms, 2048^2 4.38 -> 2.53 ms, 1024^2 1.58 ->
 // 1.15 ms, 512^2 0.82 -> 0.68 ms.
 #pragma once
+#include "sweep_batch.cuh"
 #include "sweep_mom.cuh"
 
 namespace biot {
@@ -78,14 +79,11 @@ __device__ __forceinline__ F2 from_east(F2 a)
     return f2(y, __shfl_down_sync(0xffffffffu, x, 1));
 }
 
-constexpr int PAIR_WARPS = 4;              // warps of a CTA, one strip each
-// Resident CTAs per SM that the register bound leaves room for (166 registers), and
-// rows of a ring.  Measured, ms per step at 2048^2 / 4096^2: 3 CTAs with 3, 4, 5, 6
+// Rows of a ring, at the PAIR_CTAS = 3 resident CTAs per SM that 166 registers leave
+// room for.  Measured, ms per step at 2048^2 / 4096^2: 3 CTAs with 3, 4, 5, 6
 // slots 2.53 / 7.68, 2.57 / 7.73, 2.60 / 7.68, 2.63 / 7.70 (a smaller ring leaves L1
 // to the lines that neighbouring strips share); 4 CTAs spill (4.19 / 16.6).
-constexpr int PAIR_CTAS = 3, PAIR_SLOTS = 3;
-constexpr int PAIR_COLS = 60;              // columns a strip writes: 64 less two on each side
-constexpr int PAIR_FX = 16, PAIR_FY = 2;   // frame tiles along the top and bottom; the sides take them transposed
+constexpr int PAIR_SLOTS = 3;
 static_assert(TileShape<PAIR_FX, PAIR_FY>::NT == 32 * PAIR_WARPS && TileShape<PAIR_FY, PAIR_FX>::NT == 32 * PAIR_WARPS,
               "a frame tile is one CTA");
 
@@ -388,36 +386,52 @@ __device__ __forceinline__ void sweep_pair_strip(const SweepArgs<float, TC> &a, 
     }
 }
 
-// CTAs 0 .. frame-1: tiles of the frame; the others: PAIR_WARPS strips each, row
-// blocks of TY rows, nsx strips side by side.
+// CTA b of a level's sweep: PAIR_WARPS strips, or past the strips a tile of the
+// frame.  The frame's tiles come last, where they fill the tail (first in the grid
+// they hold every SM for some 8 us: 8.68 instead of 8.13 ms per 4096^2 step).
 template <typename TC, int KIND, bool LO, bool RESTRICT, int FM>
-__global__ void __launch_bounds__(32 * PAIR_WARPS, PAIR_CTAS) k_sweep_pair(const SweepArgs<float, TC> a, int TY, int nsx, int frame)
+__device__ __forceinline__ void sweep_pair_cta(const SweepArgs<float, TC> &a, int b, int TY, unsigned char *smem,
+                                               double (&red)[3][PAIR_WARPS])
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    // the frame's tiles come last in the grid, where they fill the tail (first in the
-    // grid they hold every SM for some 8 us: 8.68 instead of 8.13 ms per 4096^2 step)
-    const int bid = blockIdx.x + frame < gridDim.x ? blockIdx.x + frame : blockIdx.x + frame - gridDim.x;
-    if (bid < frame) {
-        __shared__ double red[3][PAIR_WARPS];
+    const int strips = pair_strip_ctas(a.nx, a.ny, TY);
+    if (b >= strips) {
         const int ntx = (a.nx + PAIR_FX - 1) / PAIR_FX, nty = (a.ny + PAIR_FX - 1) / PAIR_FX;
-        int b = bid;
+        b -= strips;
         if (b < 2 * ntx) {
             const int top = b >= ntx ? 1 : 0;
-            tile_body<float, TC, PAIR_FX, PAIR_FY, KIND, LO, RESTRICT>(a, b - top * ntx, top * (a.ny / PAIR_FY - 1), smem_raw, red);
+            tile_body<float, TC, PAIR_FX, PAIR_FY, KIND, LO, RESTRICT>(a, b - top * ntx, top * (a.ny / PAIR_FY - 1), smem, red);
         } else {
             b -= 2 * ntx;
             const int right = b >= nty ? 1 : 0;
-            tile_body<float, TC, PAIR_FY, PAIR_FX, KIND, LO, RESTRICT>(a, right * (a.nx / PAIR_FY - 1), b - right * nty, smem_raw,
-                                                                      red, PAIR_FY, a.ny - PAIR_FY);
+            tile_body<float, TC, PAIR_FY, PAIR_FX, KIND, LO, RESTRICT>(a, right * (a.nx / PAIR_FY - 1), b - right * nty, smem, red,
+                                                                      PAIR_FY, a.ny - PAIR_FY);
         }
         return;
     }
     using R = PairRing<KIND, LO, FM>;
-    const int w = (bid - frame) * PAIR_WARPS + (int)(threadIdx.x >> 5);
+    const int nsx = pair_strips_x(a.nx), w = b * PAIR_WARPS + (int)(threadIdx.x >> 5);
     const int by = w / nsx, y0 = 2 + by * TY;
     if (y0 >= a.ny - 2) return;
-    float *ring = reinterpret_cast<float *>(smem_raw) + (threadIdx.x >> 5) * (R::SLOTS * R::ROW);
+    float *ring = reinterpret_cast<float *>(smem) + (threadIdx.x >> 5) * (R::SLOTS * R::ROW);
     sweep_pair_strip<TC, KIND, LO, RESTRICT, FM>(a, 2 + PAIR_COLS * (w - by * nsx), y0, min(y0 + TY, a.ny - 2), ring);
+}
+
+template <typename TC, int KIND, bool LO, bool RESTRICT, int FM>
+__global__ void __launch_bounds__(32 * PAIR_WARPS, PAIR_CTAS) k_sweep_pair(const SweepArgs<float, TC> a, int TY)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double red[3][PAIR_WARPS];
+    sweep_pair_cta<TC, KIND, LO, RESTRICT, FM>(a, blockIdx.x, TY, smem_raw, red);
+}
+
+// Batched form: the sweeps of many instances' levels, job j's CTAs start[j] ..
+template <typename TC, int KIND, bool LO, bool RESTRICT, int FM>
+__global__ void __launch_bounds__(32 * PAIR_WARPS, PAIR_CTAS) k_sweep_pair_batch(const __grid_constant__ BatchParams<float, TC> P)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double red[3][PAIR_WARPS];
+    const int j = batch_job(P, blockIdx.x);
+    sweep_pair_cta<TC, KIND, LO, RESTRICT, FM>(P.job[j], blockIdx.x - P.start[j], P.ty[j], smem_raw, red);
 }
 
 // Whether the packed sweep takes these arguments: an FP32 level without ghost
@@ -431,30 +445,73 @@ bool pair_takes(const SweepArgs<float, TC> &a)
            !(a.zero_init && a.gc) && !(a.gc && sizeof(TC) != 4) && !(a.zero_init && a.Ft);
 }
 
+// Shared memory of a CTA, and the warps of a kernel resident on the device.
+template <int KIND, bool LO, int FM>
+constexpr size_t pair_smem()
+{
+    constexpr size_t t0 = tile_smem_bytes<float, PAIR_FX, PAIR_FY, KIND, LO>(), t1 = tile_smem_bytes<float, PAIR_FY, PAIR_FX, KIND, LO>();
+    constexpr size_t t = t0 > t1 ? t0 : t1;
+    return PairRing<KIND, LO, FM>::bytes > t ? PairRing<KIND, LO, FM>::bytes : t;
+}
+template <typename K>
+cudaError_t pair_slots(K kern, size_t smem, int *slots)
+{
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int dev = 0, sms = 0, per_sm = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * PAIR_WARPS, smem);
+    if (e == cudaSuccess) *slots = sms * (per_sm > 0 ? per_sm : 1) * PAIR_WARPS;
+    return e;
+}
+
 template <typename TC, int KIND, bool LO, bool RESTRICT, int FM>
 cudaError_t launch_pair_fm(const SweepArgs<float, TC> &a, cudaStream_t s)
 {
-    constexpr size_t tile = tile_smem_bytes<float, PAIR_FX, PAIR_FY, KIND, LO>() > tile_smem_bytes<float, PAIR_FY, PAIR_FX, KIND, LO>()
-                                ? tile_smem_bytes<float, PAIR_FX, PAIR_FY, KIND, LO>()
-                                : tile_smem_bytes<float, PAIR_FY, PAIR_FX, KIND, LO>();
-    constexpr size_t smem = PairRing<KIND, LO, FM>::bytes > tile ? PairRing<KIND, LO, FM>::bytes : tile;
+    constexpr size_t smem = pair_smem<KIND, LO, FM>();
     auto kern = k_sweep_pair<TC, KIND, LO, RESTRICT, FM>;
-    static int slots = 0;  // resident warps on the device
+    static int slots = 0;
     if (!slots) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = pair_slots(kern, smem, &slots);
         if (e != cudaSuccess) return e;
-        int dev = 0, sms = 0, per_sm = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * PAIR_WARPS, smem)) != cudaSuccess) return e;
-        slots = sms * (per_sm > 0 ? per_sm : 1) * PAIR_WARPS;
     }
-    const int nsx = (a.nx - 4 + PAIR_COLS - 1) / PAIR_COLS, rows = a.ny - 4;
-    const int ty = pair_rows(nsx, rows, slots);
-    const int strips = nsx * ((rows + ty - 1) / ty);
-    const int frame = 2 * ((a.nx + PAIR_FX - 1) / PAIR_FX) + 2 * ((a.ny + PAIR_FX - 1) / PAIR_FX);
-    kern<<<frame + (strips + PAIR_WARPS - 1) / PAIR_WARPS, 32 * PAIR_WARPS, smem, s>>>(a, ty, nsx, frame);
+    const int ty = pair_rows(pair_strips_x(a.nx), a.ny - 4, slots);
+    kern<<<pair_strip_ctas(a.nx, a.ny, ty) + pair_frame_ctas(a.nx, a.ny), 32 * PAIR_WARPS, smem, s>>>(a, ty);
     return cudaGetLastError();
+}
+
+template <typename TC, int KIND, bool LO, bool RESTRICT, int FM>
+cudaError_t launch_pair_batch_fm(const BatchParams<float, TC> &P, cudaStream_t s)
+{
+    constexpr size_t smem = pair_smem<KIND, LO, FM>();
+    auto kern = k_sweep_pair_batch<TC, KIND, LO, RESTRICT, FM>;
+    static int slots = 0;
+    if (!slots) {
+        cudaError_t e = pair_slots(kern, smem, &slots);
+        if (e != cudaSuccess) return e;
+    }
+    for (int j = 0; j < P.njobs; j++)  // what the plan assumed of its jobs
+        if (!pair_takes(P.job[j]) || (FM == FETCH_PROL) != (P.job[j].gc != nullptr) || (FM == FETCH_ZERO) != (P.job[j].zero_init != 0) ||
+            P.start[j + 1] - P.start[j] != pair_strip_ctas(P.job[j].nx, P.job[j].ny, P.ty[j]) + pair_frame_ctas(P.job[j].nx, P.job[j].ny))
+            return cudaErrorInvalidValue;
+    kern<<<P.start[P.njobs], 32 * PAIR_WARPS, smem, s>>>(P);
+    return cudaGetLastError();
+}
+
+// A batched launch of storage kind v (SWEEP_V_PAIR set): FP32 levels above FP32 levels.
+inline cudaError_t launch_pair_batch(int v, const BatchParams<float, float> &P, cudaStream_t s)
+{
+    constexpr int F = KIND_FINE | KIND_NOGHOST, C = KIND_COARSE | KIND_NOGHOST;
+    const bool prol = v & SWEEP_V_PROL, zero = v & SWEEP_V_ZERO;
+    if (v & SWEEP_V_COARSE) {
+        if (v & SWEEP_V_RESTRICT) return launch_pair_batch_fm<float, C, false, true, FETCH_PLAIN>(P, s);
+        if (zero) return launch_pair_batch_fm<float, C, false, false, FETCH_ZERO>(P, s);
+        if (prol) return launch_pair_batch_fm<float, C, false, false, FETCH_PROL>(P, s);
+        return launch_pair_batch_fm<float, C, false, false, FETCH_PLAIN>(P, s);
+    }
+    if (v & SWEEP_V_RESTRICT) return launch_pair_batch_fm<float, F, true, true, FETCH_PLAIN>(P, s);
+    if (prol) return launch_pair_batch_fm<float, F, true, false, FETCH_PROL>(P, s);
+    return launch_pair_batch_fm<float, F, true, false, FETCH_PLAIN>(P, s);
 }
 
 template <typename TC, int KIND, bool LO, bool RESTRICT>
