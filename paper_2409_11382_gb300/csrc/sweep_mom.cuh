@@ -1342,13 +1342,20 @@ template <> struct TileFor<double> { static constexpr int X = 8, Y = 2; };
 static_assert(TileFor<float>::X == 32 && TileFor<float>::Y == 8 && TileFor<double>::X == 8 && TileFor<double>::Y == 2,
               "tile shapes shared with the host planner (sweep_tile_shape)");
 
+// FP64 levels from this many cells on take 16 x 8 tiles.  One FP64 instruction holds
+// its SM sub-partition for 64 clocks whatever its active lanes, and an 8 x 2 tile
+// issues about 15 per cell (its warps are mostly halo), a 16 x 8 tile 5.5: 256^2
+// FP64 2.76 -> 1.69 ms per step, 128^2 1.12 -> 0.86 ms.  32 x 8 and 16 x 16 tiles leave
+// SMs idle (1.72 and 1.80 ms at 256^2, 0.98 and 1.01 ms at 128^2), strips 1.82 ms at
+// 256^2; below 128^2 the small tiles reach more SMs (64^2: 0.57 ms, 0.63 ms with 16 x 8).
+constexpr long TILE64_LARGE_CELLS = 128L * 128L;
+
 // Levels of at most this many cells use the tile sweep.
 inline long sweep_tile_max_cells() { return SWEEP_TILE_CELLS; }
 
-template <typename T, typename TC, int KIND, bool LO, bool RESTRICT>
-cudaError_t launch_tile(const SweepArgs<T, TC> &a, cudaStream_t s)
+template <typename T, typename TC, int KIND, bool LO, bool RESTRICT, int TX, int TY>
+cudaError_t launch_tile_shape(const SweepArgs<T, TC> &a, cudaStream_t s)
 {
-    constexpr int TX = TileFor<T>::X, TY = TileFor<T>::Y;
     constexpr size_t smem = tile_smem_bytes<T, TX, TY, KIND, LO>();
     auto kern = k_sweep_tile<T, TC, TX, TY, KIND, LO, RESTRICT>;
     static bool configured = false;
@@ -1360,6 +1367,15 @@ cudaError_t launch_tile(const SweepArgs<T, TC> &a, cudaStream_t s)
     dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY);
     kern<<<grid, TileShape<TX, TY>::NT, smem, s>>>(a);
     return cudaGetLastError();
+}
+
+template <typename T, typename TC, int KIND, bool LO, bool RESTRICT>
+cudaError_t launch_tile(const SweepArgs<T, TC> &a, cudaStream_t s)
+{
+    if constexpr (sizeof(T) == 8) {
+        if ((long)a.nx * a.ny >= TILE64_LARGE_CELLS) return launch_tile_shape<T, TC, KIND, LO, RESTRICT, 16, 8>(a, s);
+    }
+    return launch_tile_shape<T, TC, KIND, LO, RESTRICT, TileFor<T>::X, TileFor<T>::Y>(a, s);
 }
 
 // Strip sweep launch shape: SWEEP_NT threads, SWEEP_CPT cells of a row per
