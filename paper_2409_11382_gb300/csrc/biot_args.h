@@ -77,9 +77,10 @@ struct SweepItem {
 // Storage kind of a sweep launch (bit flags).
 enum { SWEEP_V_COARSE = 1, SWEEP_V_LO = 2, SWEEP_V_RESTRICT = 4, SWEEP_V_NOGHOST = 8, SWEEP_V_TILE = 16,
        SWEEP_V_DEV16 = 32, SWEEP_V_DEVBF16 = 64, SWEEP_V_RESIDENT = 128,
-       // packed strips (sweep_pair.cuh), with the prolongated correction added or from zero
-       SWEEP_V_PAIR = 256, SWEEP_V_PROL = 512, SWEEP_V_ZERO = 1024,
-       SWEEP_V_SHAPE = SWEEP_V_TILE | SWEEP_V_PAIR | SWEEP_V_PROL | SWEEP_V_ZERO };  // chosen by the plan, not by the sweep
+       // packed strips (sweep_pair.cuh), with the prolongated correction added, from
+       // zero, or measuring the residual
+       SWEEP_V_PAIR = 256, SWEEP_V_PROL = 512, SWEEP_V_ZERO = 1024, SWEEP_V_MEAS = 2048,
+       SWEEP_V_SHAPE = SWEEP_V_TILE | SWEEP_V_PAIR | SWEEP_V_PROL | SWEEP_V_ZERO | SWEEP_V_MEAS };  // chosen by the plan, not by the sweep
 // Tile sweeps: levels of at most SWEEP_TILE_CELLS cells (single instance); tile
 // shape per storage type.  The fused flow step works on FLOW_TILE_X x FLOW_TILE_Y tiles.
 constexpr long SWEEP_TILE_CELLS = 256L * 256L;

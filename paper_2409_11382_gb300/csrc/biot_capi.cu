@@ -1982,13 +1982,13 @@ int op_variant(const biot_ctx *h, const PlanOp &o)
     if (o.resident) return SWEEP_V_RESIDENT | (h->P.ne_fixed > 0 ? SWEEP_V_NOGHOST : 0);
     const int v = level_variant(h, o.level, o.mode);
     // packed strips where they take the sweep (pair_takes): FP32 above FP32, double-float
-    // first moments on the finest level only, no deviation store, no measured residual
+    // first moments on the finest level only, no deviation store
     const Level &Lv = h->lv[o.level];
     const bool fine = o.level == h->L - 1;
-    const bool pair = !(v & (SWEEP_V_TILE | SWEEP_V_DEV16 | SWEEP_V_DEVBF16)) && (v & SWEEP_V_NOGHOST) && !o.measured &&
+    const bool pair = !(v & (SWEEP_V_TILE | SWEEP_V_DEV16 | SWEEP_V_DEVBF16)) && (v & SWEEP_V_NOGHOST) &&
                       level_tkind(h, o.level) == 2 && ((v & SWEEP_V_LO) != 0) == fine && Lv.nx % 4 == 0 && Lv.ny % 2 == 0 &&
                       Lv.nx >= 64 && Lv.ny >= 8;
-    return pair ? v | SWEEP_V_PAIR | o.fetch : v;
+    return pair ? v | SWEEP_V_PAIR | o.fetch | (o.measured ? SWEEP_V_MEAS : 0) : v;
 }
 
 // Strip heights of one batched launch (levels of nx x ny cells): the fewest whole

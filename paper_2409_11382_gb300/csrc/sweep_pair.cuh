@@ -116,7 +116,8 @@ __device__ __forceinline__ void pair_copy4(unsigned dst, const TC *src, bool in)
 }
 
 // Rows y0 .. y1-1 of columns x0 .. x0 + 59 (x0 = 2 mod 4, away from the sides).
-template <typename TC, int KIND, bool LO, bool RESTRICT, int FM>
+// MEAS: also the residual norms of the solve's last sweep (a.resmax).
+template <typename TC, int KIND, bool LO, bool RESTRICT, int FM, bool MEAS>
 __device__ __forceinline__ void sweep_pair_strip(const SweepArgs<float, TC> &a, int x0, int y0, int y1, float *ring)
 {
     using R = PairRing<KIND, LO, FM>;
@@ -243,6 +244,8 @@ __device__ __forceinline__ void sweep_pair_strip(const SweepArgs<float, TC> &a, 
     F2 S0, A0;                        // pair 0 of row j-1
     F2 pg1, ph1, pg4, ph4, pg5, ph5;  // the pulls into row j-1, from row j-2
     F2 acc[5];
+    float rmax = 0.0f, gmax = 0.0f;
+    double rsum = 0.0;
     take_row(P);  // row y0-2: only its m_s
     sS = ms_of(P.m[3]);
     take_row(B);
@@ -344,6 +347,20 @@ __device__ __forceinline__ void sweep_pair_strip(const SweepArgs<float, TC> &a, 
                         o[k] = mad_rn(ngam, d[k], P.m[k]);
                     }
                 }
+                if (MEAS && writes) {  // per cell, as the general strips
+                    float dc[2][8] = {}, gc[2][8] = {};
+#pragma unroll
+                    for (int k = 0; k < 5; k++) {
+                        f2_split(d[k], dc[0][k], dc[1][k]);
+                        f2_split(P.m[k], gc[0][k], gc[1][k]);
+                    }
+#pragma unroll
+                    for (int c = 0; c < 2; c++) {
+                        rmax = fmaxf(rmax, pop_absmax(dc[c]));
+                        gmax = fmaxf(gmax, pop_absmax(gc[c]));
+                        rsum += (double)pop_sumsq(dc[c]);
+                    }
+                }
                 if (writes) {
                     const size_t idx = (size_t)y * nx + x;
                     float *go = a.gout + idx;
@@ -384,12 +401,25 @@ __device__ __forceinline__ void sweep_pair_strip(const SweepArgs<float, TC> &a, 
         sS = sO;
         sO = sN;
     }
+    if constexpr (MEAS) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+            gmax = fmaxf(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
+            rsum += __shfl_xor_sync(0xffffffffu, rsum, o);
+        }
+        if (lane == 0) {
+            atomicMax(&a.resmax[0], (unsigned long long)__double_as_longlong((double)rmax));
+            atomicMax(&a.resmax[1], (unsigned long long)__double_as_longlong((double)gmax));
+            atomicAdd(reinterpret_cast<double *>(&a.resmax[2]), rsum);
+        }
+    }
 }
 
 // CTA b of a level's sweep: PAIR_WARPS strips, or past the strips a tile of the
 // frame.  The frame's tiles come last, where they fill the tail (first in the grid
 // they hold every SM for some 8 us: 8.68 instead of 8.13 ms per 4096^2 step).
-template <typename TC, int KIND, bool LO, bool RESTRICT, int FM>
+template <typename TC, int KIND, bool LO, bool RESTRICT, int FM, bool MEAS>
 __device__ __forceinline__ void sweep_pair_cta(const SweepArgs<float, TC> &a, int b, int TY, unsigned char *smem,
                                                double (&red)[3][PAIR_WARPS])
 {
@@ -413,35 +443,34 @@ __device__ __forceinline__ void sweep_pair_cta(const SweepArgs<float, TC> &a, in
     const int by = w / nsx, y0 = 2 + by * TY;
     if (y0 >= a.ny - 2) return;
     float *ring = reinterpret_cast<float *>(smem) + (threadIdx.x >> 5) * (R::SLOTS * R::ROW);
-    sweep_pair_strip<TC, KIND, LO, RESTRICT, FM>(a, 2 + PAIR_COLS * (w - by * nsx), y0, min(y0 + TY, a.ny - 2), ring);
+    sweep_pair_strip<TC, KIND, LO, RESTRICT, FM, MEAS>(a, 2 + PAIR_COLS * (w - by * nsx), y0, min(y0 + TY, a.ny - 2), ring);
 }
 
-template <typename TC, int KIND, bool LO, bool RESTRICT, int FM>
+template <typename TC, int KIND, bool LO, bool RESTRICT, int FM, bool MEAS>
 __global__ void __launch_bounds__(32 * PAIR_WARPS, PAIR_CTAS) k_sweep_pair(const SweepArgs<float, TC> a, int TY)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[3][PAIR_WARPS];
-    sweep_pair_cta<TC, KIND, LO, RESTRICT, FM>(a, blockIdx.x, TY, smem_raw, red);
+    sweep_pair_cta<TC, KIND, LO, RESTRICT, FM, MEAS>(a, blockIdx.x, TY, smem_raw, red);
 }
 
 // Batched form: the sweeps of many instances' levels, job j's CTAs start[j] ..
-template <typename TC, int KIND, bool LO, bool RESTRICT, int FM>
+template <typename TC, int KIND, bool LO, bool RESTRICT, int FM, bool MEAS>
 __global__ void __launch_bounds__(32 * PAIR_WARPS, PAIR_CTAS) k_sweep_pair_batch(const __grid_constant__ BatchParams<float, TC> P)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[3][PAIR_WARPS];
     const int j = batch_job(P, blockIdx.x);
-    sweep_pair_cta<TC, KIND, LO, RESTRICT, FM>(P.job[j], blockIdx.x - P.start[j], P.ty[j], smem_raw, red);
+    sweep_pair_cta<TC, KIND, LO, RESTRICT, FM, MEAS>(P.job[j], blockIdx.x - P.start[j], P.ty[j], smem_raw, red);
 }
 
 // Whether the packed sweep takes these arguments: an FP32 level without ghost
-// moments or deviation store, no measured residual, rows of whole 16-byte units and
-// an even number of rows, iterate stored (with or without a prolongated
+// moments or deviation store, rows of whole 16-byte units and an even number of rows, iterate stored (with or without a prolongated
 // correction) or zero, and a level below it in FP32 when its correction is added.
 template <typename TC>
 bool pair_takes(const SweepArgs<float, TC> &a)
 {
-    return !a.ghosts && !a.dev && !a.resmax && a.nx % 4 == 0 && a.ny % 2 == 0 && a.nx >= 64 && a.ny >= 8 &&
+    return !a.ghosts && !a.dev && a.nx % 4 == 0 && a.ny % 2 == 0 && a.nx >= 64 && a.ny >= 8 &&
            !(a.zero_init && a.gc) && !(a.gc && sizeof(TC) != 4) && !(a.zero_init && a.Ft);
 }
 
@@ -465,11 +494,11 @@ cudaError_t pair_slots(K kern, size_t smem, int *slots)
     return e;
 }
 
-template <typename TC, int KIND, bool LO, bool RESTRICT, int FM>
+template <typename TC, int KIND, bool LO, bool RESTRICT, int FM, bool MEAS = false>
 cudaError_t launch_pair_fm(const SweepArgs<float, TC> &a, cudaStream_t s)
 {
     constexpr size_t smem = pair_smem<KIND, LO, FM>();
-    auto kern = k_sweep_pair<TC, KIND, LO, RESTRICT, FM>;
+    auto kern = k_sweep_pair<TC, KIND, LO, RESTRICT, FM, MEAS>;
     static int slots = 0;
     if (!slots) {
         cudaError_t e = pair_slots(kern, smem, &slots);
@@ -480,38 +509,22 @@ cudaError_t launch_pair_fm(const SweepArgs<float, TC> &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-template <typename TC, int KIND, bool LO, bool RESTRICT, int FM>
+template <typename TC, int KIND, bool LO, bool RESTRICT, int FM, bool MEAS = false>
 cudaError_t launch_pair_batch_fm(const BatchParams<float, TC> &P, cudaStream_t s)
 {
     constexpr size_t smem = pair_smem<KIND, LO, FM>();
-    auto kern = k_sweep_pair_batch<TC, KIND, LO, RESTRICT, FM>;
+    auto kern = k_sweep_pair_batch<TC, KIND, LO, RESTRICT, FM, MEAS>;
     static int slots = 0;
     if (!slots) {
         cudaError_t e = pair_slots(kern, smem, &slots);
         if (e != cudaSuccess) return e;
     }
     for (int j = 0; j < P.njobs; j++)  // what the plan assumed of its jobs
-        if (!pair_takes(P.job[j]) || (FM == FETCH_PROL) != (P.job[j].gc != nullptr) || (FM == FETCH_ZERO) != (P.job[j].zero_init != 0) ||
+        if (!pair_takes(P.job[j]) || MEAS != (P.job[j].resmax != nullptr) || (FM == FETCH_PROL) != (P.job[j].gc != nullptr) || (FM == FETCH_ZERO) != (P.job[j].zero_init != 0) ||
             P.start[j + 1] - P.start[j] != pair_strip_ctas(P.job[j].nx, P.job[j].ny, P.ty[j]) + pair_frame_ctas(P.job[j].nx, P.job[j].ny))
             return cudaErrorInvalidValue;
     kern<<<P.start[P.njobs], 32 * PAIR_WARPS, smem, s>>>(P);
     return cudaGetLastError();
-}
-
-// A batched launch of storage kind v (SWEEP_V_PAIR set): FP32 levels above FP32 levels.
-inline cudaError_t launch_pair_batch(int v, const BatchParams<float, float> &P, cudaStream_t s)
-{
-    constexpr int F = KIND_FINE | KIND_NOGHOST, C = KIND_COARSE | KIND_NOGHOST;
-    const bool prol = v & SWEEP_V_PROL, zero = v & SWEEP_V_ZERO;
-    if (v & SWEEP_V_COARSE) {
-        if (v & SWEEP_V_RESTRICT) return launch_pair_batch_fm<float, C, false, true, FETCH_PLAIN>(P, s);
-        if (zero) return launch_pair_batch_fm<float, C, false, false, FETCH_ZERO>(P, s);
-        if (prol) return launch_pair_batch_fm<float, C, false, false, FETCH_PROL>(P, s);
-        return launch_pair_batch_fm<float, C, false, false, FETCH_PLAIN>(P, s);
-    }
-    if (v & SWEEP_V_RESTRICT) return launch_pair_batch_fm<float, F, true, true, FETCH_PLAIN>(P, s);
-    if (prol) return launch_pair_batch_fm<float, F, true, false, FETCH_PROL>(P, s);
-    return launch_pair_batch_fm<float, F, true, false, FETCH_PLAIN>(P, s);
 }
 
 template <typename TC, int KIND, bool LO, bool RESTRICT>
@@ -519,6 +532,12 @@ cudaError_t launch_pair(const SweepArgs<float, TC> &a, cudaStream_t s)
 {
     if constexpr (!kind_fine(KIND)) {
         if (a.zero_init) return launch_pair_fm<TC, KIND, LO, RESTRICT, FETCH_ZERO>(a, s);
+    }
+    if constexpr (kind_fine(KIND) && !RESTRICT) {
+        if constexpr (sizeof(TC) == 4) {
+            if (a.resmax && a.gc) return launch_pair_fm<TC, KIND, LO, RESTRICT, FETCH_PROL, true>(a, s);
+        }
+        if (a.resmax) return launch_pair_fm<TC, KIND, LO, RESTRICT, FETCH_PLAIN, true>(a, s);
     }
     if constexpr (sizeof(TC) == 4 && !RESTRICT) {
         if (a.gc) return launch_pair_fm<TC, KIND, LO, RESTRICT, FETCH_PROL>(a, s);
