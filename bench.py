@@ -487,7 +487,8 @@ def run_ours(args):
     avg_sweep_ms = sweep_ms / max(sweep_n, 1)
     achieved = bytes_per_cell * cells / (avg_sweep_ms / 1e3) / 1e9
     traffic_pc = profiled_traffic_per_cell(PROFILE64 if fp64 else PROFILE)
-    hbm_roof = {"kernel": f"k_sweep_mom<{'double,double' if fp64 else 'float,float'}> finest level, smoothing",
+    kernel = "k_sweep_mom<double,double>" if fp64 else "k_sweep_mom<float,float>" if dev else "k_sweep_pair<float>"
+    hbm_roof = {"kernel": f"{kernel} finest level, smoothing",
                 "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "peak_kind": f"{peak_kind} copy bandwidth (burst)",
                 "bytes_per_cell": bytes_per_cell, "launches": sweep_n, "avg_launch_ms": avg_sweep_ms,
