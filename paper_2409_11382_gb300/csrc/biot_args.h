@@ -282,6 +282,15 @@ inline int sweep_strip_rows(int nx, int ny, int slots)
         if (ty <= cap || waves >= 64) return (int)ty;
     }
 }
+// Whether packed strips (sweep_pair.cuh) take the sweeps of an FP32 level: no ghost
+// moments (fixed V-cycles), no deviation store, double-float first moments on the
+// finest level and on no other, rows of whole 16-byte units, an even number of rows
+// and at least one strip inside the frame.  The one statement of the rule: the
+// launches (pair_takes) and the plan of a batch (op_variant) both ask it.
+constexpr bool pair_takes_level(bool fine, bool lo, bool ghosts, bool dev, int nx, int ny)
+{
+    return !ghosts && !dev && lo == fine && nx % 4 == 0 && ny % 2 == 0 && nx >= 64 && ny >= 8;
+}
 // Rows per strip of the packed sweep (sweep_pair.cuh): nsx strips side by side over
 // `rows` rows, `slots` resident warps.  Whole waves of strips, as few as give strips
 // of at most 64 rows: a strip's four extra rows cost least when it is tall, and one

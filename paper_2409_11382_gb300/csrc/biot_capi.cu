@@ -1981,13 +1981,11 @@ int op_variant(const biot_ctx *h, const PlanOp &o)
 {
     if (o.resident) return SWEEP_V_RESIDENT | (h->P.ne_fixed > 0 ? SWEEP_V_NOGHOST : 0);
     const int v = level_variant(h, o.level, o.mode);
-    // packed strips where they take the sweep (pair_takes): FP32 above FP32, double-float
-    // first moments on the finest level only, no deviation store
     const Level &Lv = h->lv[o.level];
-    const bool fine = o.level == h->L - 1;
-    const bool pair = !(v & (SWEEP_V_TILE | SWEEP_V_DEV16 | SWEEP_V_DEVBF16)) && (v & SWEEP_V_NOGHOST) &&
-                      level_tkind(h, o.level) == 2 && ((v & SWEEP_V_LO) != 0) == fine && Lv.nx % 4 == 0 && Lv.ny % 2 == 0 &&
-                      Lv.nx >= 64 && Lv.ny >= 8;
+    // packed strips: FP32 levels above an FP32 one
+    const bool pair = !(v & SWEEP_V_TILE) && level_tkind(h, o.level) == 2 &&
+                      pair_takes_level(!(v & SWEEP_V_COARSE), v & SWEEP_V_LO, !(v & SWEEP_V_NOGHOST),
+                                       v & (SWEEP_V_DEV16 | SWEEP_V_DEVBF16), Lv.nx, Lv.ny);
     return pair ? v | SWEEP_V_PAIR | o.fetch | (o.measured ? SWEEP_V_MEAS : 0) : v;
 }
 

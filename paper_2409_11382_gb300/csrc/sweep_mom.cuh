@@ -1413,14 +1413,14 @@ struct SweepKernel {
 // The packed strip sweep (sweep_pair.cuh), for levels from 256^2 cells on: at 256^2
 // 0.487 ms per step against 0.501 ms with tiles, at 128^2 0.496 (too few strips).
 constexpr long PAIR_MIN_CELLS = 256L * 256L;
-template <typename TC> bool pair_takes(const SweepArgs<float, TC> &a);
+template <typename TC, int KIND, bool LO> bool pair_takes(const SweepArgs<float, TC> &a);
 template <typename TC, int KIND, bool LO, bool RESTRICT> cudaError_t launch_pair(const SweepArgs<float, TC> &a, cudaStream_t s);
 
 template <typename T, typename TC, int KIND, bool LO, bool RESTRICT>
 cudaError_t launch_rows(const SweepArgs<T, TC> &a, cudaStream_t s)
 {
-    if constexpr (sizeof(T) == 4 && !kind_ghosts(KIND) && !kind_dev(KIND) && LO == kind_fine(KIND)) {
-        if ((long)a.nx * a.ny >= PAIR_MIN_CELLS && pair_takes<TC>(a)) return launch_pair<TC, KIND, LO, RESTRICT>(a, s);
+    if constexpr (sizeof(T) == 4 && pair_takes_level(kind_fine(KIND), LO, kind_ghosts(KIND), kind_dev(KIND), 64, 8)) {
+        if ((long)a.nx * a.ny >= PAIR_MIN_CELLS && pair_takes<TC, KIND, LO>(a)) return launch_pair<TC, KIND, LO, RESTRICT>(a, s);
     }
     if ((long)a.nx * a.ny <= sweep_tile_max_cells()) return launch_tile<T, TC, KIND, LO, RESTRICT>(a, s);
     using SK = SweepKernel<T, TC, KIND, LO, RESTRICT>;

@@ -464,14 +464,14 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, PAIR_CTAS) k_sweep_pair_batch
     sweep_pair_cta<TC, KIND, LO, RESTRICT, FM, MEAS>(P.job[j], blockIdx.x - P.start[j], P.ty[j], smem_raw, red);
 }
 
-// Whether the packed sweep takes these arguments: an FP32 level without ghost
-// moments or deviation store, rows of whole 16-byte units and an even number of rows, iterate stored (with or without a prolongated
-// correction) or zero, and a level below it in FP32 when its correction is added.
-template <typename TC>
+// Whether the packed sweep takes these arguments: a level of pair_takes_level, its
+// iterate stored (with or without a prolongated correction) or zero, and a level
+// below it in FP32 when its correction is added.
+template <typename TC, int KIND, bool LO>
 bool pair_takes(const SweepArgs<float, TC> &a)
 {
-    return !a.ghosts && !a.dev && a.nx % 4 == 0 && a.ny % 2 == 0 && a.nx >= 64 && a.ny >= 8 &&
-           !(a.zero_init && a.gc) && !(a.gc && sizeof(TC) != 4) && !(a.zero_init && a.Ft);
+    return pair_takes_level(kind_fine(KIND), LO, a.ghosts != 0, a.dev != 0, a.nx, a.ny) && !(a.zero_init && a.gc) &&
+           !(a.gc && sizeof(TC) != 4) && !(a.zero_init && a.Ft);
 }
 
 // Shared memory of a CTA, and the warps of a kernel resident on the device.
@@ -520,7 +520,7 @@ cudaError_t launch_pair_batch_fm(const BatchParams<float, TC> &P, cudaStream_t s
         if (e != cudaSuccess) return e;
     }
     for (int j = 0; j < P.njobs; j++)  // what the plan assumed of its jobs
-        if (!pair_takes(P.job[j]) || MEAS != (P.job[j].resmax != nullptr) || (FM == FETCH_PROL) != (P.job[j].gc != nullptr) || (FM == FETCH_ZERO) != (P.job[j].zero_init != 0) ||
+        if (!pair_takes<TC, KIND, LO>(P.job[j]) || MEAS != (P.job[j].resmax != nullptr) || (FM == FETCH_PROL) != (P.job[j].gc != nullptr) || (FM == FETCH_ZERO) != (P.job[j].zero_init != 0) ||
             P.start[j + 1] - P.start[j] != pair_strip_ctas(P.job[j].nx, P.job[j].ny, P.ty[j]) + pair_frame_ctas(P.job[j].nx, P.job[j].ny))
             return cudaErrorInvalidValue;
     kern<<<P.start[P.njobs], 32 * PAIR_WARPS, smem, s>>>(P);
