@@ -7,7 +7,47 @@
 #include <stdint.h>
 #include <stdlib.h>
 
+#include <atomic>
+
 namespace biot {
+
+// A positive number worked out once per device -- the resident CTAs of a kernel,
+// with the attributes set on the way -- by whichever thread launches first.  Threads
+// that meet here compute the same number and store it twice; a device beyond the
+// table computes it on each call.  find() returns the number, 0 when it fails.
+struct DeviceCache {
+    static constexpr int DEVICES = 16;
+    std::atomic<int> v[DEVICES] = {};
+    template <typename F>
+    int get(F find)
+    {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+        if (dev >= DEVICES) return find(dev);
+        int n = v[dev].load(std::memory_order_acquire);
+        if (n == 0) {
+            n = find(dev);
+            v[dev].store(n, std::memory_order_release);
+        }
+        return n;
+    }
+};
+// Lets kernel k use smem bytes of dynamic shared memory and returns its resident CTAs
+// of `threads` threads over device dev (0: an error, left for cudaGetLastError).
+inline int resident_ctas(int dev, const void *k, int threads, size_t smem)
+{
+    int sms = 0, per_sm = 0;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem) != cudaSuccess) return 0;
+    return sms * (per_sm > 0 ? per_sm : 1);
+}
+// The error of a launch whose resident CTAs could not be found.
+inline cudaError_t no_slots()
+{
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : cudaErrorInvalidConfiguration;
+}
 
 enum { SIDE_BOTTOM = 0, SIDE_RIGHT = 1, SIDE_TOP = 2, SIDE_LEFT = 3 };
 enum { BC_PERIODIC = 0, BC_SYMMETRY = 1, BC_DIRICHLET = 2, BC_NEUMANN = 3 };

@@ -2,8 +2,6 @@
 // FP64 levels in one kernel.  Compiled with --fmad=false: the shared sweep
 // arithmetic writes every multiply-add it wants fused, and the FP64 levels must
 // round as in the FP64 unit.
-#include <atomic>
-
 #include "sweep_resident.cuh"
 
 cudaError_t biot::launch_resident(const biot::ResParams &P, size_t smem, cudaStream_t s)
@@ -15,18 +13,16 @@ cudaError_t biot::launch_resident(const biot::ResParams &P, size_t smem, cudaStr
 
 int biot::resident_max_cluster()
 {
-    static std::atomic<int> found{0};
-    int n = found.load();
-    if (n) return n;
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute at[1];
-    int clusters = 0;
-    n = RES_CLUSTER_MAX;
-    if (resident_config<true>(cfg, at[0], 1, n, RES_SMEM_MAX, nullptr) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&clusters, k_resident_cycle<true>, &cfg) != cudaSuccess || clusters < 1) {
+    static DeviceCache found;
+    const int n = found.get([](int) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at[1];
+        int clusters = 0;
+        if (resident_config<true>(cfg, at[0], 1, RES_CLUSTER_MAX, RES_SMEM_MAX, nullptr) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, k_resident_cycle<true>, &cfg) == cudaSuccess && clusters > 0)
+            return RES_CLUSTER_MAX;
         cudaGetLastError();
-        n = 8;
-    }
-    found.store(n);
-    return n;
+        return 8;
+    });
+    return n ? n : 8;
 }

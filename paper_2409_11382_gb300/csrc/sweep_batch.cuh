@@ -55,12 +55,11 @@ cudaError_t launch_tile_batch(const BatchParams<T, TC> &P, cudaStream_t s)
     constexpr int TX = TileFor<T>::X, TY = TileFor<T>::Y;
     constexpr size_t smem = tile_smem_bytes<T, TX, TY, KIND, LO>();
     auto kern = k_sweep_tile_batch<T, TC, TX, TY, KIND, LO, RESTRICT>;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static DeviceCache configured;
+    if (!configured.get([&](int) {
+            return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess ? 1 : 0;
+        }))
+        return no_slots();
     const int n = P.start[P.njobs];
     if (n <= 0) return cudaSuccess;
     kern<<<n, TileShape<TX, TY>::NT, smem, s>>>(P);
@@ -80,17 +79,10 @@ struct BatchKernel {
     static constexpr size_t smem = rows_smem_bytes<T, KIND, LO, BATCH_NT>();
     static int slots()
     {
-        static int n = 0;
-        if (!n) {
-            auto k = k_sweep_batch<T, TC, BATCH_NT, 1, KIND, LO, RESTRICT>;
-            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
-            int dev = 0, sms = 0, per_sm = 0;
-            if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-            if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, BATCH_NT, smem) != cudaSuccess) return 0;
-            n = sms * (per_sm > 0 ? per_sm : 1);
-        }
-        return n;
+        static DeviceCache n;
+        return n.get([](int dev) {
+            return resident_ctas(dev, (const void *)k_sweep_batch<T, TC, BATCH_NT, 1, KIND, LO, RESTRICT>, BATCH_NT, smem);
+        });
     }
 };
 

@@ -1358,12 +1358,11 @@ cudaError_t launch_tile_shape(const SweepArgs<T, TC> &a, cudaStream_t s)
 {
     constexpr size_t smem = tile_smem_bytes<T, TX, TY, KIND, LO>();
     auto kern = k_sweep_tile<T, TC, TX, TY, KIND, LO, RESTRICT>;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static DeviceCache configured;
+    if (!configured.get([&](int) {
+            return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess ? 1 : 0;
+        }))
+        return no_slots();
     dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY);
     kern<<<grid, TileShape<TX, TY>::NT, smem, s>>>(a);
     return cudaGetLastError();
@@ -1395,18 +1394,12 @@ struct SweepKernel {
     // fetch forms share one shape, and the plain form's occupancy stands for all
     static int slots()
     {
-        static int n = 0;
-        if (!n) {
-            for (auto k : {kernel<FETCH_PLAIN>(), kernel<FETCH_PROL>(), kernel<FETCH_ZERO>(), kernel<FETCH_ZPROL>()})
+        static DeviceCache n;
+        return n.get([](int dev) {
+            for (auto k : {kernel<FETCH_PROL>(), kernel<FETCH_ZERO>(), kernel<FETCH_ZPROL>()})
                 if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
-            int dev = 0, sms = 0, per_sm = 0;
-            if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-            if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel<FETCH_PLAIN>(), SWEEP_NT, smem) != cudaSuccess)
-                return 0;
-            n = sms * (per_sm > 0 ? per_sm : 1);
-        }
-        return n;
+            return resident_ctas(dev, (const void *)kernel<FETCH_PLAIN>(), SWEEP_NT, smem);
+        });
     }
 };
 

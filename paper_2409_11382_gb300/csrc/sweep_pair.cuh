@@ -474,7 +474,7 @@ bool pair_takes(const SweepArgs<float, TC> &a)
            !(a.gc && sizeof(TC) != 4) && !(a.zero_init && a.Ft);
 }
 
-// Shared memory of a CTA, and the warps of a kernel resident on the device.
+// Shared memory of a CTA.
 template <int KIND, bool LO, int FM>
 constexpr size_t pair_smem()
 {
@@ -482,29 +482,15 @@ constexpr size_t pair_smem()
     constexpr size_t t = t0 > t1 ? t0 : t1;
     return PairRing<KIND, LO, FM>::bytes > t ? PairRing<KIND, LO, FM>::bytes : t;
 }
-template <typename K>
-cudaError_t pair_slots(K kern, size_t smem, int *slots)
-{
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int dev = 0, sms = 0, per_sm = 0;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * PAIR_WARPS, smem);
-    if (e == cudaSuccess) *slots = sms * (per_sm > 0 ? per_sm : 1) * PAIR_WARPS;
-    return e;
-}
-
 template <typename TC, int KIND, bool LO, bool RESTRICT, int FM, bool MEAS = false>
 cudaError_t launch_pair_fm(const SweepArgs<float, TC> &a, cudaStream_t s)
 {
     constexpr size_t smem = pair_smem<KIND, LO, FM>();
     auto kern = k_sweep_pair<TC, KIND, LO, RESTRICT, FM, MEAS>;
-    static int slots = 0;
-    if (!slots) {
-        cudaError_t e = pair_slots(kern, smem, &slots);
-        if (e != cudaSuccess) return e;
-    }
-    const int ty = pair_rows(pair_strips_x(a.nx), a.ny - 4, slots);
+    static DeviceCache ctas;
+    const int n = ctas.get([&](int dev) { return resident_ctas(dev, (const void *)kern, 32 * PAIR_WARPS, smem); });
+    if (!n) return no_slots();
+    const int ty = pair_rows(pair_strips_x(a.nx), a.ny - 4, n * PAIR_WARPS);
     kern<<<pair_strip_ctas(a.nx, a.ny, ty) + pair_frame_ctas(a.nx, a.ny), 32 * PAIR_WARPS, smem, s>>>(a, ty);
     return cudaGetLastError();
 }
@@ -514,11 +500,9 @@ cudaError_t launch_pair_batch_fm(const BatchParams<float, TC> &P, cudaStream_t s
 {
     constexpr size_t smem = pair_smem<KIND, LO, FM>();
     auto kern = k_sweep_pair_batch<TC, KIND, LO, RESTRICT, FM, MEAS>;
-    static int slots = 0;
-    if (!slots) {
-        cudaError_t e = pair_slots(kern, smem, &slots);
-        if (e != cudaSuccess) return e;
-    }
+    static DeviceCache ctas;
+    const int n = ctas.get([&](int dev) { return resident_ctas(dev, (const void *)kern, 32 * PAIR_WARPS, smem); });
+    if (!n) return no_slots();
     for (int j = 0; j < P.njobs; j++)  // what the plan assumed of its jobs
         if (!pair_takes<TC, KIND, LO>(P.job[j]) || MEAS != (P.job[j].resmax != nullptr) || (FM == FETCH_PROL) != (P.job[j].gc != nullptr) || (FM == FETCH_ZERO) != (P.job[j].zero_init != 0) ||
             P.start[j + 1] - P.start[j] != pair_strip_ctas(P.job[j].nx, P.job[j].ny, P.ty[j]) + pair_frame_ctas(P.job[j].nx, P.job[j].ny))

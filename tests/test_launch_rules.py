@@ -79,3 +79,62 @@ def test_strips_and_frame_cover_the_level_once(tmp_path, slots):
         assert strips == -(-nsx * blocks // warps)
         # two rows at the top and bottom, two columns at the sides, tiles of fx cells along them
         assert frame == 2 * -(-nx // fx) + 2 * -(-ny // fx)
+
+
+def test_launch_code_keeps_no_plain_statics():
+    """Instances are created and stepped from several threads (a server's worker among
+    them), and a process may use several devices: what launch code remembers from its
+    first launch is atomic and per device (DeviceCache), never a plain static."""
+    plain = []
+    for name in sorted(os.listdir(CSRC)):
+        for i, line in enumerate(open(os.path.join(CSRC, name)), 1):
+            if re.match(r"\s+static (?!const|constexpr|inline|DeviceCache|std::atomic)[\w:<>]+ \*?\w+( = [^;(]*)?;", line):
+                plain.append(f"{name}:{i}: {line.strip()}")
+    assert not plain, plain
+
+
+def test_device_cache_is_one_number_per_device_from_many_threads(tmp_path):
+    src = tmp_path / "cache.cpp"
+    src.write_text(r"""
+#include "biot_args.h"
+#include <stdio.h>
+#include <thread>
+#include <vector>
+static thread_local int current = 0;
+extern "C" cudaError_t cudaGetDevice(int *d) { *d = current; return cudaSuccess; }
+int main()
+{
+    static biot::DeviceCache c, failing;
+    std::atomic<int> wrong{0}, calls{0};
+    std::vector<std::thread> t;
+    for (int i = 0; i < 16; i++)
+        t.emplace_back([&, i] {
+            for (int k = 0; k < 20000; k++) {
+                current = (i + k) % (biot::DeviceCache::DEVICES + 2);  // two beyond the table
+                if (c.get([&](int dev) { calls++; return 100 + dev; }) != 100 + current) wrong++;
+            }
+        });
+    for (auto &x : t) x.join();
+    current = 3;
+    const int f0 = failing.get([](int) { return 0; }), f1 = failing.get([](int) { return 7; });  // a failure is tried again
+    printf("%d %d %d %d\n", wrong.load(), calls.load() >= biot::DeviceCache::DEVICES, f0, f1);
+    return 0;
+}
+""")
+    from paper_2409_11382_gb300 import build as B
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B.nvcc()))), "include")
+    exe = tmp_path / "cache"
+    # under the thread sanitizer: a race in the cache ends the program with an error.  The
+    # CUDA calls that the header's other functions name are never made here
+    cmd = ["g++", "-std=c++17", "-O1", "-g", "-pthread", f"-I{CSRC}", f"-I{cuda}", str(src), "-o", str(exe),
+           "-Wl,--unresolved-symbols=ignore-all"]
+
+    def run(extra):
+        if subprocess.run(cmd + extra, capture_output=True).returncode:
+            return None
+        return subprocess.run([str(exe)], capture_output=True, text=True)
+    out = run(["-fsanitize=thread"])
+    if out is None or "unexpected memory mapping" in out.stderr:  # no sanitizer on this host
+        out = run([])
+    assert out is not None and out.returncode == 0, out and out.stderr[-2000:]
+    assert out.stdout.split() == ["0", "1", "0", "7"]
