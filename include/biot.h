@@ -306,9 +306,7 @@ BIOT_API int biot_load(biot_handle h, const void *buf, size_t size);
  * strips (more than 256^2 cells) and both sweep modes (smoothing, residual +
  * restriction), time candidate strip heights (4 .. 96 rows) on a scratch
  * instance of the same shape (allocated for the call, then freed) and keep
- * the fastest for this instance.  (FP32 sweeps that run as packed strips choose
- * their height by a rule of their own; the tuned heights serve the others.)
- * Strip heights do not change the arithmetic:
+ * the fastest for this instance.  Strip heights do not change the arithmetic:
  * results are bitwise the same as untuned.  rows_out / ms_out (may be NULL)
  * receive 2 values per level (smoothing, restriction; level 0 = coarsest) for
  * the first max_levels levels: the rows chosen (0 = not tuned) and the mean

@@ -354,6 +354,13 @@ inline int pair_rows(int nsx, int rows, int slots)
         if (ty <= 64 || waves >= 64) return ty;
     }
 }
+// The height of a launch: biot_autotune's choice for the level (tuned > 0, made even,
+// at least one strip step of four rows), else the rule's.
+inline int pair_height(int tuned, int nsx, int rows, int slots)
+{
+    if (tuned <= 0) return pair_rows(nsx, rows, slots);
+    return tuned < 4 ? 4 : tuned + (tuned & 1);
+}
 // CTAs of the strips of an nx x ny level in row blocks of TY rows, and of its frame.
 __host__ __device__ inline int pair_strips_x(int nx) { return (nx - 4 + PAIR_COLS - 1) / PAIR_COLS; }
 __host__ __device__ inline int pair_strip_ctas(int nx, int ny, int TY)

@@ -1972,6 +1972,14 @@ int level_variant(const biot_ctx *h, int l, int mode)
            (tile ? SWEEP_V_TILE : 0) | (fine && h->dev == 1 ? SWEEP_V_DEV16 : 0) | (fine && h->dev == 2 ? SWEEP_V_DEVBF16 : 0);
 }
 
+// Whether packed strips take level l's sweeps of variant v (FP32 levels large enough
+// for strips).
+bool level_takes_pair(const biot_ctx *h, int l, int v)
+{
+    return !h->lv[l].fp64 && pair_takes_level(!(v & SWEEP_V_COARSE), v & SWEEP_V_LO, !(v & SWEEP_V_NOGHOST),
+                                              v & (SWEEP_V_DEV16 | SWEEP_V_DEVBF16), h->lv[l].nx, h->lv[l].ny);
+}
+
 int op_tkind(const biot_ctx *h, const PlanOp &o)
 {
     return o.resident ? 2 : level_tkind(h, o.level);
@@ -1981,11 +1989,8 @@ int op_variant(const biot_ctx *h, const PlanOp &o)
 {
     if (o.resident) return SWEEP_V_RESIDENT | (h->P.ne_fixed > 0 ? SWEEP_V_NOGHOST : 0);
     const int v = level_variant(h, o.level, o.mode);
-    const Level &Lv = h->lv[o.level];
     // packed strips: FP32 levels above an FP32 one
-    const bool pair = !(v & SWEEP_V_TILE) && level_tkind(h, o.level) == 2 &&
-                      pair_takes_level(!(v & SWEEP_V_COARSE), v & SWEEP_V_LO, !(v & SWEEP_V_NOGHOST),
-                                       v & (SWEEP_V_DEV16 | SWEEP_V_DEVBF16), Lv.nx, Lv.ny);
+    const bool pair = !(v & SWEEP_V_TILE) && level_tkind(h, o.level) == 2 && level_takes_pair(h, o.level, v);
     return pair ? v | SWEEP_V_PAIR | o.fetch | (o.measured ? SWEEP_V_MEAS : 0) : v;
 }
 
@@ -3242,6 +3247,14 @@ extern "C" int biot_autotune(biot_handle h, int *rows_out, double *ms_out, int m
         release(c);
         return fail(BIOT_ERR_CUDA, "cudaEventCreate failed");
     }
+    int dev = 0, sms = 1;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        release(c);
+        return fail(BIOT_ERR_CUDA, "device query failed");
+    }
     static const int fixed_cand[] = {4, 8, 16, 24, 32, 48, 64, 96};
     int status = BIOT_OK;
     for (int l = 0; l < h->L && !status; l++) {
@@ -3255,8 +3268,15 @@ extern "C" int biot_autotune(biot_handle h, int *rows_out, double *ms_out, int m
             // candidates: fixed heights, and the heights whose strips fill exactly
             // 1, 2 or 3 waves of resident CTAs (tall strips repeat fewer halo rows)
             std::vector<int> cand(std::begin(fixed_cand), std::end(fixed_cand));
-            const int slots = strips ? tkind_strip_slots(level_tkind(h, l), level_variant(h, l, mode) & ~SWEEP_V_TILE) : 0;
+            const int v = level_variant(h, l, mode) & ~SWEEP_V_TILE;
+            const bool pair = strips && level_takes_pair(h, l, v);
+            const int slots = strips && !pair ? tkind_strip_slots(level_tkind(h, l), v) : 0;
             const int sx = (Lv.nx + SWEEP_STRIP_COLS - 1) / SWEEP_STRIP_COLS;
+            if (pair) {
+                const int nsx = pair_strips_x(Lv.nx), warps = sms * PAIR_CTAS * PAIR_WARPS;
+                for (int w = 1; w <= 3; w++) cand.push_back(pair_rows_for(nsx, Lv.ny - 4, w * warps));
+                cand.push_back(pair_rows(nsx, Lv.ny - 4, warps));  // the height without tuning
+            }
             for (int w = 1; w <= 3 && slots > 0; w++) {
                 const int nsy = w * slots / sx;
                 if (nsy < 1) continue;

@@ -490,7 +490,7 @@ cudaError_t launch_pair_fm(const SweepArgs<float, TC> &a, cudaStream_t s)
     static DeviceCache ctas;
     const int n = ctas.get([&](int dev) { return resident_ctas(dev, (const void *)kern, 32 * PAIR_WARPS, smem); });
     if (!n) return no_slots();
-    const int ty = pair_rows(pair_strips_x(a.nx), a.ny - 4, n * PAIR_WARPS);
+    const int ty = pair_height(a.rows, pair_strips_x(a.nx), a.ny - 4, n * PAIR_WARPS);
     kern<<<pair_strip_ctas(a.nx, a.ny, ty) + pair_frame_ctas(a.nx, a.ny), 32 * PAIR_WARPS, smem, s>>>(a, ty);
     return cudaGetLastError();
 }

@@ -56,7 +56,8 @@ def test_plan_and_launch_ask_the_same_rule():
         text = open(os.path.join(CSRC, name)).read()
         i = text.index(start)
         return text[i:text.index("\n}\n", i)]
-    assert "pair_takes_level(" in body("biot_capi.cu", "int op_variant(const biot_ctx *h, const PlanOp &o)\n{")
+    assert "pair_takes_level(" in body("biot_capi.cu", "bool level_takes_pair(const biot_ctx *h, int l, int v)\n{")
+    assert "level_takes_pair(" in body("biot_capi.cu", "int op_variant(const biot_ctx *h, const PlanOp &o)\n{")
     assert "pair_takes_level(" in body("sweep_pair.cuh", "bool pair_takes(const SweepArgs<float, TC> &a)\n{")
     assert "pair_takes_level(" in body("sweep_mom.cuh", "cudaError_t launch_rows(")
     for name in ("biot_capi.cu", "sweep_pair.cuh", "sweep_mom.cuh"):  # and none restates it
@@ -138,3 +139,18 @@ int main()
         out = run([])
     assert out is not None and out.returncode == 0, out and out.stderr[-2000:]
     assert out.stdout.split() == ["0", "1", "0", "7"]
+
+
+def test_packed_strips_take_the_tuned_height(tmp_path):
+    """biot_autotune's height is the launch's, made even and at least four rows; without
+    one the rule's.  The launch and the candidates of the tuner are the packed form's."""
+    tuned = [0, -1, 1, 2, 3, 4, 5, 17, 64, 96, 158]
+    got = evaluate(tmp_path, [f'printf("%d %d\\n", pair_height({t}, 69, 4092, 1824), pair_rows(69, 4092, 1824));'
+                              for t in tuned])
+    for t, (height, rule) in zip(tuned, got):
+        assert height == (rule if t <= 0 else max(4, t + t % 2)), t
+    pair = open(os.path.join(CSRC, "sweep_pair.cuh")).read()
+    assert "pair_height(a.rows," in pair
+    capi = open(os.path.join(CSRC, "biot_capi.cu")).read()
+    tuner = capi[capi.index('extern "C" int biot_autotune(biot_handle h, int *rows_out'):]
+    assert "level_takes_pair(" in tuner and "pair_rows_for(" in tuner
