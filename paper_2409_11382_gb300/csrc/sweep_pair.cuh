@@ -53,9 +53,15 @@ __device__ __forceinline__ F2 mad_rn(F2 a, F2 b, F2 c)
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
     return r;
 }
-// A product.  (The assembler fuses a packed product into a packed sum that is its
-// only use, explicit rounding or not -- seen in the force below -- so such a sum is
-// written as an fma whose factor 1 it cannot know: see `one` in sweep_pair_strip.)
+// A product.  The assembler fuses a packed product into a packed sum that is its only
+// use, explicit rounding or not (seen in the force below), and then rounds once where
+// every other form of a sweep rounds twice.  The rule for every product that meets a
+// packed sum or difference: it has a second use, which keeps it a value of its own (q3,
+// q6, q7, q0, q2 meet a sum and a difference each, the coarse force four), or the sum is
+// an fma whose factor 1 the assembler cannot know (`one` in sweep_pair_strip).  A product
+// as the addend of an fma is safe, and one with -1 is exact.  Writing all of these sums
+// that way costs 0.3 to 0.7 % of a step (1024^2: 1.146 -> 1.156 ms), for nothing while the
+// results are bitwise those of the general strips, as the tests demand.
 __device__ __forceinline__ F2 mul_rn(F2 a, F2 b)
 {
     F2 r;
@@ -79,8 +85,8 @@ __device__ __forceinline__ F2 from_east(F2 a)
     return f2(y, __shfl_down_sync(0xffffffffu, x, 1));
 }
 
-// Rows of a ring, at the PAIR_CTAS = 3 resident CTAs per SM that 166 registers leave
-// room for.  Measured, ms per step at 2048^2 / 4096^2: 3 CTAs with 3, 4, 5, 6
+// Rows of a ring, at the PAIR_CTAS = 3 resident CTAs per SM that 124 to 168 registers
+// (148 for plain smoothing of the finest level) leave room for.  Measured, ms per step at 2048^2 / 4096^2: 3 CTAs with 3, 4, 5, 6
 // slots 2.53 / 7.68, 2.57 / 7.73, 2.60 / 7.68, 2.63 / 7.70 (a smaller ring leaves L1
 // to the lines that neighbouring strips share); 4 CTAs spill (4.19 / 16.6).
 constexpr int PAIR_SLOTS = 3;
