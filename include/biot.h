@@ -90,12 +90,16 @@ extern "C" {
                                          in every solve (default: in an FP32 solve at t = 0) */
 #define BIOT_OPT_COARSE_LO_OFF   16   /* ... in no solve */
 #define BIOT_OPT_SEGMENTS        32   /* a launch choice, honoured in every precision.  By default
-                                         the coarse-grid correction below a small level (64^2 cells;
-                                         16^2 in a batch) is one thread-block-cluster launch that keeps
-                                         its levels in shared memory, one cluster per instance.  With
-                                         this flag that launch starts at levels of up to four times the
-                                         cells as far as they fit, and the solve at t = 0 takes it too:
-                                         fewer launches, bitwise the same results */
+                                         the coarse-grid correction of a small level is one thread-block-
+                                         cluster launch that keeps its levels in shared memory, one
+                                         cluster per instance.  It starts at the finest coarse level of at
+                                         most 64^2 cells in FP32 (32^2 with BIOT_OPT_COARSEST_STORAGE),
+                                         2048 cells in FP64, 16^2 in a batch.  With this flag it starts at
+                                         levels of up to four times the cells as far as they fit 16 blocks
+                                         of 512 threads (single instance: 5472 cells in FP32, 66 x 64 among
+                                         the squarest; no more than by default in FP64), and the solve at t = 0 takes
+                                         it too on levels without double-float first moments: fewer
+                                         launches, bitwise the same results */
 
 /* ---- boundary condition types (§3.6) --------------------------------------- */
 #define BIOT_PERIODIC  0  /* wrap-around streaming; must be set on both opposite sides

@@ -557,10 +557,13 @@ int res_min_cells(const biot_ctx *h, bool fp64) { return !fp64 ? 256 : h->batche
 // The largest level of a resident cycle, in cells.  Single instance: up to what
 // 16 CTAs hold, 64^2 in FP32 (against 32^2: 0.457 and 0.469 ms per 128^2 step,
 // 0.528 and 0.554 ms at 256^2, 1.62 and 1.66 ms at 1024^2) and 2048 cells in FP64
-// (against 1024: 0.600 and 0.686 ms per 64^2 FP64 step); with an FP32 coarsest
-// level 32^2, where 64^2 gains 1 % (0.793 and 0.801 ms at 512^2).  A batch's phase
-// launches fill the GPU, and a cluster holds SMs that they would use: 16^2 (with
-// the general strips 6.63 ms per step of the 64-instance workload, 32^2: 6.77, 64^2: 7.75).
+// (against 1024: 0.600 and 0.686 ms per 64^2 FP64 step).  With an FP32 coarsest level
+// 32^2: its 64^2 levels take the launch with BIOT_OPT_SEGMENTS, whose promise of fewer
+// launches than the default rests on them there; with it a step is up to 8 % shorter
+// (128^2 0.345 and 0.372 ms, 512^2 0.633 and 0.657 ms, 1024^2 1.095 and 1.121 ms; 64^2 the
+// same).  A batch's phase launches fill the GPU, and a cluster holds SMs that they would
+// use: 16^2 (with the general strips 6.63 ms per step of the 64-instance workload, 32^2:
+// 6.77, 64^2: 7.75).
 long res_max_cells(const biot_ctx *h, bool fp64)
 {
     if (h->batched) return 256;
@@ -655,9 +658,12 @@ bool res_plan(const biot_ctx *h, int s, int kind, ResLaunch &R)
 // The finest level whose coarse-grid correction runs as one resident launch (-1:
 // none): every level down from it is within the bound and fits one cluster, and
 // none has double-float first moments (which the resident form does not take).
-// The solve at t = 0 runs once per instance and has them on its FP32 levels, so it
-// keeps one launch per sweep.  BIOT_OPT_SEGMENTS: levels of up to four times the
-// cells, and at t = 0 too.
+// The solve at t = 0 runs once per instance and keeps one launch per sweep: its FP32
+// levels have them (unless BIOT_OPT_COARSE_LO_OFF), which leaves it an 8^2 level or so
+// (64^2 FP32 instance: 0.70 ms with the launch, 0.86 without).  Its FP64 levels have none
+// and could take it (64^2 FP64 instance: 0.71 ms, 1.19 without).  BIOT_OPT_SEGMENTS, which
+// promises fewer launches than the default, takes it at t = 0 in both, and levels of up
+// to four times the cells.
 int res_start(const biot_ctx *h, bool cold, int kind = BIOT_CYCLE_V)
 {
     const bool more = (h->P.options & BIOT_OPT_SEGMENTS) != 0;

@@ -1348,6 +1348,8 @@ static_assert(TileFor<float>::X == 32 && TileFor<float>::Y == 8 && TileFor<doubl
 // FP64 2.76 -> 1.69 ms per step, 128^2 1.12 -> 0.86 ms.  32 x 8 and 16 x 16 tiles leave
 // SMs idle (1.72 and 1.80 ms at 256^2, 0.98 and 1.01 ms at 128^2), strips 1.82 ms at
 // 256^2; below 128^2 the small tiles reach more SMs (64^2: 0.57 ms, 0.63 ms with 16 x 8).
+// Single instances only: a batch plans its work lists with one tile per storage type
+// (sweep_tile_shape) and keeps 8 x 2 for FP64, where 16 x 8 has not been tried.
 constexpr long TILE64_LARGE_CELLS = 128L * 128L;
 
 // Levels of at most this many cells use the tile sweep.
