@@ -19,11 +19,13 @@
 // It writes the cells two or more away from every side; the frame around them --
 // the wall cells and those whose pulls see ghost values -- is done by small tiles of
 // the general code in the same launch.
-// What bounds it: HBM at 4096^2 (0.199 ms per finest sweep, 1.08 GB: 5.4 TB/s, 0.81
-// of the copy bandwidth; 0.265 ms before), and below that the latency of a row in
-// few warps (2048^2 0.094 -> 0.058 ms, 1024^2 0.034 -> 0.021 ms, 512^2 0.0175 -> 0.0123
-// ms).  Per time step: 4096^2 11.4 -> 7.7 ms, 2048^2 4.38 -> 2.53 ms, 1024^2 1.58 ->
-// 1.15 ms, 512^2 0.82 -> 0.68 ms.
+// What bounds it: HBM at 4096^2 (0.196 ms per finest sweep in the timed step, 1.08 GB:
+// 5.5 TB/s, 0.82 of the copy bandwidth), and below that the latency of a row in few
+// warps.  Against the strips it replaced, both with tuned heights: the finest sweep of a
+// step 0.248 -> 0.196 ms at 4096^2; back to back 0.238 -> 0.185 ms, 2048^2 77 -> 52 us,
+// 1024^2 27 -> 17 us, 512^2 13.4 -> 8.8 us.  Per time step (the small levels' launch and the
+// wall table are in it): 4096^2 10.6 -> 7.6 ms, 2048^2 4.0 -> 2.5 ms, 1024^2 1.89 -> 1.14 ms,
+// 512^2 1.18 -> 0.68 ms; with default heights 11.4 -> 7.6, 4.4 -> 2.5, 2.0 -> 1.15, 1.20 -> 0.69.
 #pragma once
 #include "sweep_batch.cuh"
 #include "sweep_mom.cuh"
