@@ -34,10 +34,10 @@ sys.path.insert(0, ROOT)
 
 METRIC = "MLUPS & time per Biot step at stated error vs FP64 oracle"
 WORKLOAD = "terzaghi_4097x4097_fp32"
-PROFILE = os.path.join(ROOT, "profiles", "sweep_pair_fp32_2048.md")
+PROFILE = os.path.join(ROOT, "profiles", "sweep_pair_fp32.md")
 PROFILE64 = os.path.join(ROOT, "profiles", "sweep_fp64_terzaghi_4097.md")
-KERNEL_SRC = {PROFILE: os.path.join(ROOT, "paper_2409_11382_gb300", "csrc", "sweep_pair.cuh"),
-              PROFILE64: os.path.join(ROOT, "paper_2409_11382_gb300", "csrc", "sweep_mom.cuh")}
+CSRC = os.path.join(ROOT, "paper_2409_11382_gb300", "csrc")
+KERNEL_UNIT = {PROFILE: "kernels_fp32.cu", PROFILE64: "kernels_fp64.cu"}  # the unit that holds the profiled kernel
 
 
 def dist_info():
@@ -55,14 +55,30 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
+def kernel_sources(path=PROFILE):
+    """The files that a profiled kernel's launch is built from: its unit, every
+    header that the unit includes, and the build's flags."""
+    seen, todo = [], [os.path.join(CSRC, KERNEL_UNIT[path])]
+    while todo:
+        f = todo.pop()
+        if f in seen:
+            continue
+        seen.append(f)
+        todo += [os.path.join(CSRC, inc) for inc in re.findall(r'^#include "([^"]+)"', open(f).read(), flags=re.M)]
+    return sorted(seen) + [os.path.join(ROOT, "paper_2409_11382_gb300", "build.py")]
+
+
 def kernel_sha(path=PROFILE):
-    return hashlib.sha256(open(KERNEL_SRC[path], "rb").read()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for f in kernel_sources(path):
+        h.update(open(f, "rb").read())
+    return h.hexdigest()[:16]
 
 
 def profiled_per_cell(key, path=PROFILE):
     """A per-cell figure of one finest-level sweep (``key: value``) from a
-    committed ncu summary, or None if the kernel source changed since the
-    counters were taken."""
+    committed ncu summary, or None if any source of the kernel changed since
+    the counters were taken."""
     if not os.path.exists(path):
         return None
     text = open(path).read()
@@ -73,8 +89,21 @@ def profiled_per_cell(key, path=PROFILE):
     return float(m.group(1))
 
 
-def profiled_traffic_per_cell(path=PROFILE):
-    return profiled_per_cell("traffic_bytes_per_cell", path)
+def profiled_traffic(cells, path=PROFILE):
+    """DRAM bytes of one finest-level sweep over `cells` cells, from counters taken
+    at that size: at another one a different share of the state stays in L2
+    between launches, so nothing is scaled."""
+    per_cell = profiled_per_cell("traffic_bytes_per_cell", path)
+    at = profiled_per_cell("traffic_cells", path)
+    return None if per_cell is None or at != cells else per_cell * cells
+
+
+def coarse_sweeps_label(segments, precision="fp32", batched=False):
+    """How the small coarse levels run: the bound of BIOT_OPT_SEGMENTS (biot.h)."""
+    bound = "16^2 cells" if batched else "2048 cells" if precision == "fp64" else "64^2 cells"
+    if segments:
+        return f"one cluster launch from levels above {bound} down (BIOT_OPT_SEGMENTS)"
+    return f"one cluster launch from at most {bound} down"
 
 
 DEV_PRECISIONS = {"fp32dev16": 3, "fp32devbf16": 4}  # BIOT_FP32_DEV16, BIOT_FP32_DEVBF16 of include/biot.h
@@ -488,13 +517,13 @@ def run_ours(args):
     avg_sweep_ms = sweep_ms / max(sweep_n, 1)
     achieved = bytes_per_cell * cells / (avg_sweep_ms / 1e3) / 1e9
     # (the deviation store runs the general strips, which the FP32 summary does not cover)
-    traffic_pc = None if dev else profiled_traffic_per_cell(PROFILE64 if fp64 else PROFILE)
+    traffic = None if dev else profiled_traffic(cells, PROFILE64 if fp64 else PROFILE)
     kernel = "k_sweep_mom<double,double>" if fp64 else "k_sweep_mom<float,float>" if dev else "k_sweep_pair<float>"
     hbm_roof = {"kernel": f"{kernel} finest level, smoothing",
                 "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "peak_kind": f"{peak_kind} copy bandwidth (burst)",
                 "bytes_per_cell": bytes_per_cell, "launches": sweep_n, "avg_launch_ms": avg_sweep_ms,
-                "traffic": None if traffic_pc is None else traffic_pc * cells}
+                "traffic": traffic}
     roofline, roofline_other = hbm_roof, None
     if fp64:
         # FP64 arithmetic: FP64 instructions per cell from the committed ncu counters
@@ -520,7 +549,7 @@ def run_ours(args):
                    "precision": precision_label(params, fp64),
                    "l2": f"state ({st['device_bytes'] / 1e9:.1f} GB) larger than L2; no flush needed",
                    "parallelism": f"replicas{world}",
-                   "coarse_sweeps": "cluster launches, BIOT_OPT_SEGMENTS" if args.segments else "cluster launches below 64^2 (batch: 16^2)",
+                   "coarse_sweeps": coarse_sweeps_label(args.segments, args.precision),
                    "autotuned_strip_rows": tuned},
         "roofline": roofline,
         "cpu_baseline": cpu_base,
@@ -688,7 +717,7 @@ def run_batched(args):
                        "cells_total": cells, "ne_fixed": 3, "K": 4,
                        "l2": "state of all instances larger than L2; no flush needed",
                        "parallelism": f"replicas{world}",
-                       "coarse_sweeps": "cluster launches, BIOT_OPT_SEGMENTS" if args.segments else "cluster launches below 64^2 (batch: 16^2)",
+                       "coarse_sweeps": coarse_sweeps_label(args.segments, batched=True),
                        "launches_per_step": st["launches_per_step"]},
             "e2e": {"value": cells * e2e_steps / e2e / 1e6, "unit": "MLUPS",
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h // e2e_steps,
